@@ -9,7 +9,7 @@
 // leaf of largest surface area, up to 7 of them, and the binary topology over
 // those leaves of least surface-area cost,
 //     c(S) = C_node A(S) + min over splits S = P + (S \ P) of c(P) + c(S \ P),
-// is found by dynamic programming over the 127 subsets, one warp per treelet.
+// is found by dynamic programming over the 127 subsets, eight lanes per treelet.
 // When it is cheaper the treelet is rewired with its own internal nodes.  The
 // leaves are finally renumbered in depth-first order so that every subtree's
 // triangles are contiguous again (the 8-wide collapse relies on that).
@@ -17,18 +17,30 @@
 
 namespace {
 
-constexpr int kBlock = 128;             // 4 warps, each with its own shared treelet workspace
+constexpr int kBlock = 128;             // 4 warps (32 threads a block: 2 % slower rebuild)
 constexpr int kWarps = kBlock / 32;
 constexpr int kTreelet = 7;             // treelet leaves
 constexpr int kSubsets = 1 << kTreelet;
+constexpr int kGroup = 8;               // lanes that work on one treelet
+constexpr int kGroups = 32 / kGroup;    // treelets a warp works on at a time
 constexpr float kCostNode = 1.2f;       // surface-area cost of visiting a node ...
 constexpr float kCostTri = 1.0f;        // ... and of testing a triangle
 constexpr int kMaxWalk = 256;
 
+// Half the surface area of a box, every rounding written out: the restructured
+// tree must not depend on how a compiler contracts these sums in one place or
+// another (an ulp decides between two topologies of nearly equal cost).
 __device__ __forceinline__ float half_area(float4 lo, float4 hi)
 {
-    const float dx = hi.x - lo.x, dy = hi.y - lo.y, dz = hi.z - lo.z;
-    return dx * dy + dy * dz + dz * dx;
+    const float dx = __fsub_rn(hi.x, lo.x), dy = __fsub_rn(hi.y, lo.y), dz = __fsub_rn(hi.z, lo.z);
+    return __fmaf_rn(dz, dx, __fmaf_rn(dx, dy, __fmul_rn(dy, dz)));
+}
+
+// the same for the subsets that the dynamic program compares
+__device__ __forceinline__ float subset_half_area(float4 lo, float4 hi)
+{
+    const float dx = __fsub_rn(hi.x, lo.x), dy = __fsub_rn(hi.y, lo.y), dz = __fsub_rn(hi.z, lo.z);
+    return __fmaf_rn(dz, dx, __fmaf_rn(dy, dz, __fmul_rn(dx, dy)));
 }
 
 struct Tree {
@@ -61,166 +73,310 @@ __global__ void k_cost(Tree T)
         if (atomicAdd(&T.visit[node], 1) == 0) return;
         __threadfence();
         const int2 c = __ldcg(T.child + node);
-        T.cost[node] = kCostNode * half_area(__ldcg(T.nlo + node), __ldcg(T.nhi + node)) + ref_cost(T, c.x) +
-                       ref_cost(T, c.y);
+        T.cost[node] = __fadd_rn(__fmaf_rn(kCostNode, half_area(__ldcg(T.nlo + node), __ldcg(T.nhi + node)), ref_cost(T, c.x)),
+                                 ref_cost(T, c.y));
         __threadfence();
         node = T.par_i[node];
     }
 }
 
+// One treelet's shared memory.  Its size is 32 bytes past a multiple of 128, so
+// that the four treelets of a warp start eight banks apart.
 struct Workspace {
-    int leaf[kTreelet];          // treelet leaves (node or ~leaf references)
-    int inner[kTreelet - 1];     // the treelet's internal nodes, root first
-    float4 lo[kTreelet], hi[kTreelet];
-    float area[kSubsets];
+    float4 lo[kTreelet], hi[kTreelet];  // boxes of the treelet's leaves
+    float4 ulo[24], uhi[24];            // unions of leaves 0-2 (entries 0-7, by subset) and of leaves 3-6 (entries 8-23)
     float copt[kSubsets];
     unsigned char part[kSubsets];
-    int n;
+    int leaf[kTreelet + 1];             // treelet leaves (node or ~leaf references)
+    int inner[kTreelet + 1];            // the treelet's internal nodes, root first
+    int set[kTreelet + 1], node[kTreelet + 1], ref0[kTreelet + 1], ref1[kTreelet + 1];  // the new topology, parents first
+    int pad[32];
+};
+static_assert(sizeof(Workspace) % 128 == 32, "treelets of a warp eight banks apart");
+
+// the non-empty subsets of kTreelet leaves ordered by size, then by value: those
+// of size k among the first n leaves are the first C(n, k) of their size
+__constant__ unsigned char kBySize[kSubsets] = {
+    1, 2, 4, 8, 16, 32, 64, 3, 5, 6, 9, 10, 12, 17, 18, 20, 24, 33, 34, 36, 40, 48, 65, 66, 68, 72,
+    80, 96, 7, 11, 13, 14, 19, 21, 22, 25, 26, 28, 35, 37, 38, 41, 42, 44, 49, 50, 52, 56, 67, 69, 70, 73,
+    74, 76, 81, 82, 84, 88, 97, 98, 100, 104, 112, 15, 23, 27, 29, 30, 39, 43, 45, 46, 51, 53, 54, 57, 58, 60,
+    71, 75, 77, 78, 83, 85, 86, 89, 90, 92, 99, 101, 102, 105, 106, 108, 113, 114, 116, 120, 31, 47, 55, 59, 61, 62,
+    79, 87, 91, 93, 94, 103, 107, 109, 110, 115, 117, 118, 121, 122, 124, 63, 95, 111, 119, 123, 125, 126, 127, 0,
 };
 
-// the whole warp optimises the treelet rooted at `root`
-__device__ void optimise_treelet(const Tree& T, int root, Workspace& w)
+__host__ __device__ constexpr int choose(int n, int k)  // C(n, k), n <= 7
 {
-    const unsigned lane = threadIdx.x & 31u;
-    if (lane == 0) {
-        // grow the treelet: expand the leaf of largest area that is an internal node
-        const int2 c = __ldcg(T.child + root);
-        w.leaf[0] = c.x;
-        w.leaf[1] = c.y;
-        w.inner[0] = root;
-        int n = 2;
-        while (n < kTreelet) {
-            int best = -1;
-            float ba = -1.f;
-            for (int i = 0; i < n; ++i) {
-                if (w.leaf[i] < 0) continue;
-                const float a = half_area(ref_lo(T, w.leaf[i]), ref_hi(T, w.leaf[i]));
-                if (a > ba) { ba = a; best = i; }
+    int c = 1;
+    for (int i = 0; i < k; ++i) c = c * (n - i) / (i + 1);
+    return c;
+}
+__host__ __device__ constexpr int size_first(int k)  // position of the first subset of size k
+{
+    int at = 0;
+    for (int j = 1; j < k; ++j) at += choose(kTreelet, j);
+    return at;
+}
+
+__device__ __forceinline__ void subset_box(const Workspace& w, int S, float4& lo, float4& hi)
+{
+    const float4 a = w.ulo[S & 7], b = w.ulo[8 + (S >> 3)], c = w.uhi[S & 7], d = w.uhi[8 + (S >> 3)];
+    lo = make_float4(fminf(a.x, b.x), fminf(a.y, b.y), fminf(a.z, b.z), 0.f);
+    hi = make_float4(fmaxf(c.x, d.x), fmaxf(c.y, d.y), fmaxf(c.z, d.z), 0.f);
+}
+
+// cost of subset S from the cost of its best split
+__device__ __forceinline__ float subset_cost(const Workspace& w, int S, float split)
+{
+    float4 lo, hi;
+    subset_box(w, S, lo, hi);
+    return __fmaf_rn(kCostNode, subset_half_area(lo, hi), split);
+}
+
+// Best splits of the subsets of SIZE leaves, eight lanes over the subsets of one
+// treelet.  The number of splits is a constant, so the loads of several splits
+// are in flight together.
+template <int SIZE>
+__device__ __forceinline__ void best_splits(Workspace& w, const unsigned char* by_size, int n, int gl)
+{
+    const int count = SIZE < n ? choose(n, SIZE) : 0;
+    for (int k = gl; k < count; k += kGroup) {
+        const int S = by_size[size_first(SIZE) + k];
+        const int low = S & -S, rest = S ^ low;
+        float best = 3.4e38f;
+        int bp = low, sub = rest;
+        // P holds the lowest leaf of S, so every split is seen once
+#pragma unroll
+        for (int t = 0; t < (1 << (SIZE - 1)) - 1; ++t) {
+            sub = (sub - 1) & rest;
+            const int P = low | sub;
+            const float c = w.copt[P] + w.copt[S ^ P];
+            if (c < best) {
+                best = c;
+                bp = P;
             }
-            if (best < 0) break;
-            const int node = w.leaf[best];
-            const int2 cc = __ldcg(T.child + node);
-            w.inner[n - 1] = node;
-            w.leaf[best] = cc.x;
-            w.leaf[n] = cc.y;
+        }
+        w.copt[S] = subset_cost(w, S, best);
+        w.part[S] = (unsigned char)bp;
+    }
+    __syncwarp();
+}
+
+// Optimise up to four treelets, one per group of eight lanes (root < 0: the
+// group has none).  All 32 lanes call it.
+//
+// What bounds it: issue slots (half of them used), mostly the 966 splits of a
+// seven-leaf treelet.  One warp per treelet, with one lane growing it (about 40
+// dependent L2 reads) and one lane on the full set's 63 splits, took 7.8 ms a
+// pass over 2,050,412 triangles, nearly all of it latency.  Eight lanes hold a
+// treelet's leaves in registers and fetch each new leaf's box, cost and children
+// as soon as it is known, so growing costs one L2 latency per level; the splits
+// of the full set are shared by the group; subset boxes are the union of two
+// table entries; 2.1 to 2.4 ms a pass, the same trees.
+__device__ void optimise_treelets(const Tree& T, int root, Workspace& w, const unsigned char* by_size)
+{
+    const unsigned full_mask = 0xffffffffu;
+    const int gl = (int)(threadIdx.x & (kGroup - 1));  // lane in the group
+    const bool on = root >= 0;
+    __syncwarp();
+    // grow the treelet: expand the leaf of largest area that is an internal node
+    int n = on ? 2 : 0;
+    int ref = 0;
+    int2 kids = make_int2(0, 0);
+    float area = -1.f, cost = 0.f;
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+    auto fetch = [&](int r) {
+        ref = r;
+        lo = __ldcg(r < 0 ? T.llo + ~r : T.nlo + r);
+        hi = __ldcg(r < 0 ? T.lhi + ~r : T.nhi + r);
+        if (r >= 0) {
+            kids = __ldcg(T.child + r);
+            cost = __ldcg(T.cost + r);
+        }
+        const float a = half_area(lo, hi);
+        if (r < 0) cost = kCostTri * a;
+        area = r >= 0 ? a : -1.f;  // only internal nodes are expanded
+    };
+    if (on) {
+        const int2 c = __ldcg(T.child + root);
+        if (gl == 0) w.inner[0] = root;
+        if (gl < 2) fetch(gl == 0 ? c.x : c.y);
+    }
+    bool grow = on;
+    for (int step = 2; step < kTreelet; ++step) {
+        // the largest area of the group, the lowest lane among equals
+        float best = gl < n && area > -1.f ? area : -1.f;
+        int who = gl;
+#pragma unroll
+        for (int o = 1; o < kGroup; o <<= 1) {
+            const float b = __shfl_xor_sync(full_mask, best, o);
+            const int v = __shfl_xor_sync(full_mask, who, o);
+            if (b > best || (b == best && v < who)) {
+                best = b;
+                who = v;
+            }
+        }
+        const int node = __shfl_sync(full_mask, ref, who, kGroup);
+        const int cx = __shfl_sync(full_mask, kids.x, who, kGroup), cy = __shfl_sync(full_mask, kids.y, who, kGroup);
+        grow = grow && best > -1.f;
+        if (grow) {
+            if (gl == 0) w.inner[n - 1] = node;
+            if (gl == who || gl == n) fetch(gl == who ? cx : cy);
             ++n;
         }
-        w.n = n;
-        for (int i = 0; i < n; ++i) {
-            w.lo[i] = ref_lo(T, w.leaf[i]);
-            w.hi[i] = ref_hi(T, w.leaf[i]);
-        }
+        if (__ballot_sync(full_mask, grow) == 0) break;
+    }
+    if (gl < n) {
+        w.leaf[gl] = ref;
+        w.lo[gl] = lo;
+        w.hi[gl] = hi;
+        w.copt[1 << gl] = cost;
     }
     __syncwarp();
-    const int n = w.n;
     const int full = (1 << n) - 1;
-    // areas of all subsets, leaf costs
-    for (int S = 1 + (int)lane; S <= full; S += 32) {
-        float4 lo = make_float4(3.4e38f, 3.4e38f, 3.4e38f, 0.f), hi = make_float4(-3.4e38f, -3.4e38f, -3.4e38f, 0.f);
-        for (int i = 0; i < n; ++i) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const int e = gl + r * kGroup;
+        const int first = e < 8 ? 0 : 3, S = (e < 8 ? e : (e - 8) << 3) & full;
+        float4 a = make_float4(3.4e38f, 3.4e38f, 3.4e38f, 0.f), b = make_float4(-3.4e38f, -3.4e38f, -3.4e38f, 0.f);
+        for (int i = first; i < first + 4; ++i) {
             if (!(S & (1 << i))) continue;
-            lo = make_float4(fminf(lo.x, w.lo[i].x), fminf(lo.y, w.lo[i].y), fminf(lo.z, w.lo[i].z), 0.f);
-            hi = make_float4(fmaxf(hi.x, w.hi[i].x), fmaxf(hi.y, w.hi[i].y), fmaxf(hi.z, w.hi[i].z), 0.f);
+            const float4 l = w.lo[i], h = w.hi[i];
+            a = make_float4(fminf(a.x, l.x), fminf(a.y, l.y), fminf(a.z, l.z), 0.f);
+            b = make_float4(fmaxf(b.x, h.x), fmaxf(b.y, h.y), fmaxf(b.z, h.z), 0.f);
         }
-        w.area[S] = half_area(lo, hi);
-        if (__popc(S) == 1) w.copt[S] = ref_cost(T, w.leaf[__ffs(S) - 1]);
+        w.ulo[e] = a;
+        w.uhi[e] = b;
     }
     __syncwarp();
-    // subsets by size: the best split of each
-    for (int size = 2; size <= n; ++size) {
-        for (int S = 1 + (int)lane; S <= full; S += 32) {
-            if (__popc(S) != size) continue;
-            const int low = S & -S, rest = S ^ low;
-            float best = 3.4e38f;
-            int bp = low;
-            // P holds the lowest leaf of S, so every split is seen once
-            for (int sub = rest;; sub = (sub - 1) & rest) {
-                const int P = low | sub;
-                if (P != S) {
-                    const float c = w.copt[P] + w.copt[S ^ P];
-                    if (c < best) { best = c; bp = P; }
-                }
-                if (sub == 0) break;
-            }
-            w.copt[S] = kCostNode * w.area[S] + best;
-            w.part[S] = (unsigned char)bp;
+    // subsets by size, each by one lane: the best split of each
+    const unsigned nmax = __reduce_max_sync(full_mask, (unsigned)n);
+    if (nmax > 2) best_splits<2>(w, by_size, n, gl);
+    if (nmax > 3) best_splits<3>(w, by_size, n, gl);
+    if (nmax > 4) best_splits<4>(w, by_size, n, gl);
+    if (nmax > 5) best_splits<5>(w, by_size, n, gl);
+    if (nmax > 6) best_splits<6>(w, by_size, n, gl);
+    // the full set: its splits, shared by the lanes, in the same order (the t-th
+    // submask below `rest`); the first of the smallest wins
+    bool better = false;
+    {
+        float best = 3.4e38f;
+        int bt = 1 << kTreelet;
+        const int splits = n >= 3 ? (1 << (n - 1)) - 1 : 0;
+        for (int t = gl; t < splits; t += kGroup) {
+            const int P = full - 2 * (t + 1);
+            const float c = w.copt[P] + w.copt[full ^ P];
+            if (c < best) { best = c; bt = t; }
         }
-        __syncwarp();
+#pragma unroll
+        for (int o = 1; o < kGroup; o <<= 1) {
+            const float b = __shfl_xor_sync(full_mask, best, o);
+            const int v = __shfl_xor_sync(full_mask, bt, o);
+            if (b < best || (b == best && v < bt)) {
+                best = b;
+                bt = v;
+            }
+        }
+        if (n >= 3) {
+            const float c = subset_cost(w, full, best);
+            better = c < __ldcg(T.cost + root) * (1.f - 1e-6f);
+            if (gl == 0) w.part[full] = (unsigned char)(bt < splits ? full - 2 * (bt + 1) : 1);
+        }
     }
-    if (lane == 0 && n >= 3 && w.copt[full] < __ldcg(T.cost + root) * (1.f - 1e-6f)) {
-        // rewire: internal nodes in the order they are assigned (parents first)
-        int stack_set[kTreelet], stack_node[kTreelet], order[kTreelet - 1];
+    if (__ballot_sync(full_mask, better) == 0) return;
+    __syncwarp();
+    // rewire: internal nodes in the order they are assigned (parents first)
+    if (better && gl == 0) {
         int sp = 0, next = 1, m = 0;
+        int stack_set[kTreelet], stack_node[kTreelet];
         stack_set[sp] = full;
         stack_node[sp++] = root;
         while (sp > 0) {
             --sp;
             const int S = stack_set[sp], node = stack_node[sp];
-            order[m++] = node;
-            const int P = w.part[S], Q = S ^ P;
-            int ref[2];
-            const int sets[2] = {P, Q};
+            const int P = w.part[S];
+            int ref2[2];
             for (int side = 0; side < 2; ++side) {
-                const int X = sets[side];
+                const int X = side == 0 ? P : S ^ P;
                 if (__popc(X) == 1) {
-                    ref[side] = w.leaf[__ffs(X) - 1];
+                    ref2[side] = w.leaf[__ffs(X) - 1];
                 } else {
-                    ref[side] = w.inner[next++];
+                    ref2[side] = w.inner[next++];
                     stack_set[sp] = X;
-                    stack_node[sp++] = ref[side];
+                    stack_node[sp++] = ref2[side];
                 }
-                if (ref[side] < 0) T.par_l[~ref[side]] = node;
-                else T.par_i[ref[side]] = node;
             }
-            T.child[node] = make_int2(ref[0], ref[1]);
+            w.set[m] = S;
+            w.node[m] = node;
+            w.ref0[m] = ref2[0];
+            w.ref1[m] = ref2[1];
+            ++m;
         }
-        // boxes and costs, children before parents
+        // costs, children before parents (copt of the chosen sets becomes the nodes' cost)
         for (int i = m - 1; i >= 0; --i) {
-            const int node = order[i];
-            const int2 c = __ldcg(T.child + node);
-            const float4 l0 = ref_lo(T, c.x), h0 = ref_hi(T, c.x), l1 = ref_lo(T, c.y), h1 = ref_hi(T, c.y);
-            const float4 lo = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
-            const float4 hi = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
-            T.nlo[node] = lo;
-            T.nhi[node] = hi;
-            T.cost[node] = kCostNode * half_area(lo, hi) + ref_cost(T, c.x) + ref_cost(T, c.y);
+            const int S = w.set[i], P = w.part[S];
+            float4 lo2, hi2;
+            subset_box(w, S, lo2, hi2);
+            w.copt[S] = __fadd_rn(__fmaf_rn(kCostNode, half_area(lo2, hi2), w.copt[P]), w.copt[S ^ P]);
         }
+    }
+    __syncwarp();
+    if (better && gl < n - 1) {  // a treelet of n leaves has n - 1 internal nodes, one per lane
+        const int S = w.set[gl], node = w.node[gl], r0 = w.ref0[gl], r1 = w.ref1[gl];
+        float4 nl, nh;
+        subset_box(w, S, nl, nh);
+        T.child[node] = make_int2(r0, r1);
+        if (r0 < 0) T.par_l[~r0] = node;
+        else T.par_i[r0] = node;
+        if (r1 < 0) T.par_l[~r1] = node;
+        else T.par_i[r1] = node;
+        T.nlo[node] = nl;
+        T.nhi[node] = nh;
+        T.cost[node] = w.copt[S];
         __threadfence();
     }
     __syncwarp();
 }
 
 // one restructuring pass: leaves walk up; each node whose second child finished
-// is optimised by the warp of the thread that finished it
+// is optimised by the warp of the thread that finished it, four at a time.  A
+// node over two leaves has one topology only and is passed.
 __global__ void __launch_bounds__(kBlock) k_treelets(Tree T)
 {
-    __shared__ Workspace ws[kWarps];
-    Workspace& w = ws[threadIdx.x / 32];
-    const unsigned lane = threadIdx.x & 31u;
+    __shared__ Workspace ws[kWarps * kGroups];
+    __shared__ unsigned char by_size[kSubsets];
+    for (int i = (int)threadIdx.x; i < kSubsets; i += kBlock) by_size[i] = kBySize[i];
+    __syncthreads();
+    Workspace& w = ws[threadIdx.x / kGroup];
+    const unsigned group = (threadIdx.x & 31u) / kGroup;
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int32_t node = k < T.n_leaves ? T.par_l[k] : -1;
     bool active = node >= 0;
     for (int guard = 0; guard < kMaxWalk; ++guard) {
-        bool ready = false;
+        bool ready = false, pick = false;
         if (active) {
             if (atomicAdd(&T.visit[node], 1) == 0) active = false;  // the sibling subtree is not finished
             else ready = true;
         }
-        if (ready) __threadfence();
-        unsigned todo = __ballot_sync(0xffffffffu, ready);
+        if (ready) {
+            __threadfence();
+            const int2 c = __ldcg(T.child + node);
+            pick = c.x >= 0 || c.y >= 0;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, pick);
         if (todo == 0 && __ballot_sync(0xffffffffu, active) == 0) break;
         while (todo) {
-            const int src = __ffs(todo) - 1;
-            todo &= todo - 1;
+            unsigned mine = todo;  // this group's root: the group-th of the lanes still to do
+            for (unsigned g = 0; g < group; ++g) mine &= mine - 1;
+            const int src = mine ? __ffs(mine) - 1 : 0;
             const int root = __shfl_sync(0xffffffffu, node, src);
-            optimise_treelet(T, root, w);
+            optimise_treelets(T, mine ? root : -1, w, by_size);
+            for (int g = 0; g < kGroups; ++g) todo &= todo - 1;
         }
         if (ready) {
             node = __ldcg(T.par_i + node);
             active = node >= 0;
         }
     }
-    (void)lane;
 }
 
 // leaves (and internal nodes) in depth-first order: the position of a node's
