@@ -190,8 +190,10 @@ rt_status rt_sdf_prepare(rt_sdf* sdf, void* stream);
  * fast sweeping build (Section 3, "Distance Field Generation") by its exact
  * definition.  method: RT_BAKE_BRUTE tests every triangle for every sample
  * (triangles staged through shared memory); RT_BAKE_BVH prunes with the BVH
- * (same result up to float rounding); RT_BAKE_AUTO picks by problem size.  Writes through the
- * grid pointer given to rt_sdf_create.  On a cascade (rt_cascade_create) every
+ * (same result up to float rounding); RT_BAKE_AUTO picks by problem size: the
+ * values of RT_BAKE_BRUTE up to 2^34 pairs of a sample and a triangle (found
+ * through the BVH where that is faster), those of RT_BAKE_BVH beyond.  Writes
+ * through the grid pointer given to rt_sdf_create.  On a cascade (rt_cascade_create) every
  * level is baked at its lattice points (ilo_k + i) * h_k, each coordinate
  * rounded once from that product, so that a level moved by rt_cascade_recenter
  * holds the same values as one baked at its new place.

@@ -403,7 +403,7 @@ extern "C" rt_status rt_cascade_recenter(const rt_scene* sc, rt_sdf* sdf, const 
             rebuilt[n_rebuilt++] = k;
             continue;
         }
-        st = rt_launch_cascade_bake(sc, sdf, k, RT_BAKE_BVH, keep, shift, s);
+        st = rt_launch_cascade_bake(sc, sdf, k, keep, shift, s);
         if (st != RT_OK) return st;
         st = rt_launch_cascade_cells(sdf, k, s);
         if (st != RT_OK) return st;

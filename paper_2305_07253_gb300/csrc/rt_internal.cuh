@@ -17,7 +17,9 @@
 //            internal-mask bit set, an inner child at first child + (inner children in lower slots)
 //   wtris  : 48 B per triangle in wide-leaf order (each node's leaf triangles contiguous)
 //   pn     : 112 B per triangle in leaf order: face normal, 3 edge and 3 vertex
-//            pseudonormals (float4 each), read only by the distance bake
+//            pseudonormals (float4 each), read only by the distance bake; w of the
+//            face normal: 4e-5 of the squared longest edge, the bake's margin for its
+//            plane test (inf: a badly shaped triangle, never decided by its plane)
 //   slot   : 4 B per triangle: input index -> leaf-order position (field build)
 //   grid   : caller memory, dense n0*n1*n2 float32 or float16, x fastest
 //   cells  : optional library copy of the grid with the 8 corners of every cell
@@ -240,6 +242,12 @@ rt_status rt_launch_merge_hits(const HitEntry* list, const unsigned* count, int 
 constexpr int kConcNearBlocks = RT_CONC_NEAR_BLOCKS;
 constexpr int kConcFieldBlocks = RT_CONC_FIELD_BLOCKS;
 
+// Device scratch in stream order (free it with cudaFreeAsync).  Up to
+// kScratchKept bytes come from the library's pool, which keeps what is freed;
+// more comes from the device's default pool, which gives it back.
+constexpr size_t kScratchKept = (size_t)64 << 20;
+rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+
 // allow_concurrent = false: the stages of a closest-hit split call run in
 // sequence on s (no internal streams), as the pieces of rt_trace_combined_host need
 rt_status rt_launch_trace(const TraceArgs& a, bool counted, cudaStream_t s, StageTiming* timing = nullptr,
@@ -256,8 +264,8 @@ rt_status rt_treelet_optimise(int64_t nt, int passes, int2* child, int2* range, 
                               int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, cudaStream_t s);
 rt_status rt_fill_trace_args(TraceArgs& a, const rt_scene* sc, const rt_sdf* sdf, const rt_split_params* p);
 void rt_cascade_geometry(const rt_sdf* sdf, int k, float lo[3], float hi[3], float* h, float* ih);
-rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, int32_t method, const void* keep,
-                                 const int32_t shift[3], cudaStream_t s);
+rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, const void* keep, const int32_t shift[3],
+                                 cudaStream_t s);
 rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int k, cudaStream_t s);
 rt_status rt_launch_df_sites(const rt_scene* sc, const rt_sdf* sdf, int32_t stage, int32_t* d_sites, cudaStream_t s);
 rt_status rt_launch_df_levels(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t* jfa_store,

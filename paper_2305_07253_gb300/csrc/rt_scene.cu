@@ -265,7 +265,12 @@ __global__ void k_face_normals(const float* V, const int32_t* F, int64_t nt, flo
     float len = sqrtf(n.x * n.x + n.y * n.y + n.z * n.z);
     if (len > 0.f) n = make_float3(n.x / len, n.y / len, n.z / len);
     else n = make_float3(0.f, 0.f, 0.f);
-    fn[t] = make_float4(n.x, n.y, n.z, 0.f);
+    // margin of the bake's plane test: the direction of a normal whose edges are
+    // nearly parallel is uncertain, and such a triangle is not decided by its plane
+    const float3 e3 = make_float3(p[2].x - p[1].x, p[2].y - p[1].y, p[2].z - p[1].z);
+    const float l2 = fmaxf(fmaxf(e1.x * e1.x + e1.y * e1.y + e1.z * e1.z, e2.x * e2.x + e2.y * e2.y + e2.z * e2.z),
+                           e3.x * e3.x + e3.y * e3.y + e3.z * e3.z);
+    fn[t] = make_float4(n.x, n.y, n.z, len > 0.1f * l2 ? 4e-5f * l2 : __int_as_float(0x7f800000));
     for (int c = 0; c < 3; ++c) {
         float3 q = p[(c + 1) % 3], r = p[(c + 2) % 3];
         float3 x = make_float3(q.x - p[c].x, q.y - p[c].y, q.z - p[c].z);

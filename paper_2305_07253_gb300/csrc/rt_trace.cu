@@ -696,6 +696,20 @@ void launch_simple(const TraceArgs& a, int L, unsigned nb, int block, cudaStream
 
 std::mutex& rt_conc_mutex() { return g_conc_mu; }
 
+rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s)
+{
+    *p = nullptr;
+    if (bytes > kScratchKept) {
+        RT_CUDA_TRY(cudaMallocAsync(p, bytes, s));
+        return RT_OK;
+    }
+    DeviceInfo* dev = nullptr;
+    const rt_status st = device_info(dev);
+    if (st != RT_OK) return st;
+    RT_CUDA_TRY(cudaMallocFromPoolAsync(p, bytes, dev->pool, s));
+    return RT_OK;
+}
+
 rt_status rt_conc_streams(ConcStreams*& out)
 {
     int dev = 0;
