@@ -39,58 +39,52 @@ __device__ __forceinline__ float dot3r(const float* a, const float* b)
     return __fadd_rn(__fadd_rn(__fmul_rn(a[0], b[0]), __fmul_rn(a[1], b[1])), __fmul_rn(a[2], b[2]));
 }
 
-// squared distance from p to triangle abc (Ericson's Voronoi regions)
-__device__ float tri_d2_rn(const float* p, const float* a, const float* b, const float* c)
+// Squared distance from p to triangle abc (Ericson's Voronoi regions).  Lanes
+// mostly fall in different regions, so there are no branches: the region picks
+// the operands of one division and of q = (base + s1 dir1) + s2 dir2.  A vertex
+// has s1 = s2 = 0 and an edge s2 = 0, which leave base + s1 dir1 as it is.
+__device__ __forceinline__ float tri_d2_rn(const float* p, const float* a, const float* b, const float* c)
 {
-    float ab[3], ac[3], ap[3], q[3];
+    float ab[3], ac[3], ap[3], bp[3], cp[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         ab[k] = __fsub_rn(b[k], a[k]);
         ac[k] = __fsub_rn(c[k], a[k]);
         ap[k] = __fsub_rn(p[k], a[k]);
+        bp[k] = __fsub_rn(p[k], b[k]);
+        cp[k] = __fsub_rn(p[k], c[k]);
     }
-    const float d1 = dot3r(ab, ap), d2 = dot3r(ac, ap);
-    if (d1 <= 0.f && d2 <= 0.f) {
+    const float d1 = dot3r(ab, ap), d2 = dot3r(ac, ap), d3 = dot3r(ab, bp), d4 = dot3r(ac, bp);
+    const float d5 = dot3r(ab, cp), d6 = dot3r(ac, cp);
+    const float vc = __fsub_rn(__fmul_rn(d1, d4), __fmul_rn(d3, d2));
+    const float vb = __fsub_rn(__fmul_rn(d5, d2), __fmul_rn(d1, d6));
+    const float va = __fsub_rn(__fmul_rn(d3, d6), __fmul_rn(d5, d4));
+    const float e43 = __fsub_rn(d4, d3), e56 = __fsub_rn(d5, d6);
+    // the regions in the order they are tested; the first that holds
+    const bool at_a = d1 <= 0.f && d2 <= 0.f;
+    const bool at_b = !at_a && d3 >= 0.f && d4 <= d3;
+    const bool on_ab = !at_a && !at_b && vc <= 0.f && d1 >= 0.f && d3 <= 0.f;
+    const bool past_ab = !at_a && !at_b && !on_ab;
+    const bool at_c = past_ab && d6 >= 0.f && d5 <= d6;
+    const bool on_ac = past_ab && !at_c && vb <= 0.f && d2 >= 0.f && d6 <= 0.f;
+    const bool on_bc = past_ab && !at_c && !on_ac && va <= 0.f && e43 >= 0.f && e56 >= 0.f;
+    const bool vertex = at_a || at_b || at_c, face = past_ab && !at_c && !on_ac && !on_bc;
+    const float num = vertex ? 0.f : (on_ab ? d1 : (on_ac ? d2 : (on_bc ? e43 : 1.f)));
+    const float den = vertex ? 1.f
+                             : (on_ab ? __fsub_rn(d1, d3)
+                                      : (on_ac ? __fsub_rn(d2, d6)
+                                               : (on_bc ? __fadd_rn(e43, e56) : __fadd_rn(__fadd_rn(va, vb), vc))));
+    const float r = __fdiv_rn(num, den);
+    const float s1 = face ? __fmul_rn(vb, r) : r, s2 = face ? __fmul_rn(vc, r) : 0.f;
+    const bool from_b = at_b || on_bc;
+    float pq[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) q[k] = a[k];
-    } else {
-        float bp[3], cp[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            bp[k] = __fsub_rn(p[k], b[k]);
-            cp[k] = __fsub_rn(p[k], c[k]);
-        }
-        const float d3 = dot3r(ab, bp), d4 = dot3r(ac, bp);
-        const float vc = __fsub_rn(__fmul_rn(d1, d4), __fmul_rn(d3, d2));
-        const float d5 = dot3r(ab, cp), d6 = dot3r(ac, cp);
-        const float vb = __fsub_rn(__fmul_rn(d5, d2), __fmul_rn(d1, d6));
-        const float va = __fsub_rn(__fmul_rn(d3, d6), __fmul_rn(d5, d4));
-        if (d3 >= 0.f && d4 <= d3) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = b[k];
-        } else if (vc <= 0.f && d1 >= 0.f && d3 <= 0.f) {
-            const float s = __fdiv_rn(d1, __fsub_rn(d1, d3));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = __fadd_rn(a[k], __fmul_rn(s, ab[k]));
-        } else if (d6 >= 0.f && d5 <= d6) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = c[k];
-        } else if (vb <= 0.f && d2 >= 0.f && d6 <= 0.f) {
-            const float s = __fdiv_rn(d2, __fsub_rn(d2, d6));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = __fadd_rn(a[k], __fmul_rn(s, ac[k]));
-        } else if (va <= 0.f && __fsub_rn(d4, d3) >= 0.f && __fsub_rn(d5, d6) >= 0.f) {
-            const float s = __fdiv_rn(__fsub_rn(d4, d3), __fadd_rn(__fsub_rn(d4, d3), __fsub_rn(d5, d6)));
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = __fadd_rn(b[k], __fmul_rn(s, __fsub_rn(c[k], b[k])));
-        } else {
-            const float den = __fdiv_rn(1.f, __fadd_rn(__fadd_rn(va, vb), vc));
-            const float v = __fmul_rn(vb, den), w = __fmul_rn(vc, den);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) q[k] = __fadd_rn(__fadd_rn(a[k], __fmul_rn(ab[k], v)), __fmul_rn(ac[k], w));
-        }
+    for (int k = 0; k < 3; ++k) {
+        const float base = from_b ? b[k] : (at_c ? c[k] : a[k]);
+        const float dir = on_ac ? ac[k] : (on_bc ? __fsub_rn(c[k], b[k]) : ab[k]);
+        const float q = __fadd_rn(__fadd_rn(base, __fmul_rn(s1, dir)), __fmul_rn(s2, ac[k]));
+        pq[k] = __fsub_rn(p[k], q);
     }
-    const float pq[3] = {__fsub_rn(p[0], q[0]), __fsub_rn(p[1], q[1]), __fsub_rn(p[2], q[2])};
     return dot3r(pq, pq);
 }
 
@@ -164,44 +158,55 @@ __device__ __forceinline__ void df_pos(const DfGrid& g, int64_t i, int64_t j, in
         p[a] = g.lattice ? __fmul_rn((float)(g.ilo[a] + ii[a]), g.h[a]) : __fmaf_rn((float)ii[a], g.h[a], g.lo[a]);
 }
 
+// Inside a build a site is a position in leaf order, so that a candidate's
+// triangle is one load away; "best" compares input indices, which come with the
+// triangle.  Sites that leave a build (rt_sdf_sites, the seeds of finer levels)
+// are input indices.
 struct Tris {
-    const float4* tris;   // leaf order, 3 per triangle
+    const float4* tris;   // leaf order, 3 per triangle: v0.xyz | input index, v1.xyz, v2.xyz
     const int32_t* slot;  // input index -> leaf position
     int64_t n;
 };
 
-__device__ __forceinline__ void tri_verts(const Tris& T, int32_t t, float* A, float* B, float* C)
+struct TriV {
+    float a[3], b[3], c[3];
+    int32_t id;  // input index
+};
+
+__device__ __forceinline__ TriV tri_verts(const Tris& T, int32_t k)
 {
-    const int64_t k = 3 * (int64_t)__ldg(T.slot + t);
-    const float4 a = __ldg(T.tris + k), b = __ldg(T.tris + k + 1), c = __ldg(T.tris + k + 2);
-    A[0] = a.x; A[1] = a.y; A[2] = a.z;
-    B[0] = b.x; B[1] = b.y; B[2] = b.z;
-    C[0] = c.x; C[1] = c.y; C[2] = c.z;
+    const float4* p = T.tris + 3 * (int64_t)k;
+    const float4 a = __ldg(p), b = __ldg(p + 1), c = __ldg(p + 2);
+    return {{a.x, a.y, a.z}, {b.x, b.y, b.z}, {c.x, c.y, c.z}, __float_as_int(a.w)};
 }
 
-__device__ __forceinline__ float site_d2(const Tris& T, const float* p, int32_t t)
+// the better of two (squared distance, input index); id < 0: none
+__device__ __forceinline__ bool site_better(float d2, int32_t id, float cur_d2, int32_t cur_id)
 {
-    float A[3], B[3], C[3];
-    tri_verts(T, t, A, B, C);
-    return tri_d2_rn(p, A, B, C);
+    return cur_id < 0 || d2 < cur_d2 || (d2 == cur_d2 && id < cur_id);
 }
 
-// keep the better of (cur, cur_d2) and candidate t
-__device__ __forceinline__ void site_consider(const Tris& T, const float* p, int32_t t, int32_t& cur, float& cur_d2)
+// Whether the triangle's box alone shows that tri_d2_rn(p, t) > d2.  The margins
+// (4e-5 of d2, and the square of 1.4e-4 of the position, whose ulp rounds the
+// closest point) are well above the roundings of both sides.
+__device__ __forceinline__ bool tri_farther(const float* p, const TriV& t, float d2)
 {
-    if (t < 0 || t == cur) return;
-    const float d2 = site_d2(T, p, t);
-    if (cur < 0 || d2 < cur_d2 || (d2 == cur_d2 && t < cur)) {
-        cur = t;
-        cur_d2 = d2;
+    float lb = 0.f, pp = 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float lo = rtdev::min3f(t.a[k], t.b[k], t.c[k]), hi = rtdev::max3f(t.a[k], t.b[k], t.c[k]);
+        const float e = rtdev::max3f(lo - p[k], p[k] - hi, 0.f);
+        lb = fmaf(e, e, lb);
+        pp = fmaf(p[k], p[k], pp);
     }
+    return lb > fmaf(4e-5f, d2, d2) + 2e-8f * pp;
 }
 
 // samples whose voxels the triangle's bounds may reach: the range is widened by
 // a small fraction of a voxel, far more than the rounding of the sample
 // positions, and the separating-axis test decides
 __device__ __forceinline__ bool tri_range(const DfGrid& g, const float* A, const float* B, const float* C,
-                                          int64_t r0[3], int64_t r1[3])
+                                          int32_t r0[3], int32_t r1[3])
 {
     bool empty = false;
 #pragma unroll
@@ -211,8 +216,8 @@ __device__ __forceinline__ bool tri_range(const DfGrid& g, const float* A, const
         const float x0f = ceilf((lo_t - g.origin_f[a] - g.margin[a]) * g.ih_f[a]);
         const float x1f = floorf((hi_t - g.origin_f[a] + g.margin[a]) * g.ih_f[a]);
         // clamp in float first: far-away triangles give values beyond the int range
-        const int64_t x0 = (int64_t)fmaxf(x0f, 0.f);
-        const int64_t x1 = (int64_t)fminf(x1f, (float)(g.n[a] - 1));
+        const int32_t x0 = (int32_t)fminf(fmaxf(x0f, 0.f), (float)g.n[a]);
+        const int32_t x1 = (int32_t)fmaxf(fminf(x1f, (float)(g.n[a] - 1)), -1.f);
         r0[a] = x0;
         r1[a] = x1;
         empty = empty || x0 > x1 || x1f < 0.f || x0f > (float)(g.n[a] - 1);
@@ -220,16 +225,21 @@ __device__ __forceinline__ bool tri_range(const DfGrid& g, const float* A, const
     return !empty;
 }
 
-// test one (triangle, sample) pair and keep the better site of the sample
-__device__ __forceinline__ void vox_pair(const DfGrid& g, int32_t t, const float* A, const float* B, const float* C,
-                                         int64_t i, int64_t j, int64_t k, unsigned long long* keys)
+// Test one (triangle, sample) pair and keep the better site of the sample.  On a
+// coarse level thousands of triangles share a voxel: a pair that is no better
+// than what the sample has needs neither the separating axes nor the atomic.
+__device__ __forceinline__ void vox_pair(const DfGrid& g, const TriV& t, int32_t i, int32_t j, int32_t k,
+                                         unsigned long long* keys)
 {
     float p[3];
     df_pos(g, i, j, k, p);
-    if (!tri_box(p, g.hs, A, B, C)) return;
-    const float d2 = tri_d2_rn(p, A, B, C);
-    const unsigned long long key = ((unsigned long long)__float_as_uint(d2) << 32) | (uint32_t)t;
-    atomicMin(keys + i + (int64_t)g.n[0] * (j + (int64_t)g.n[1] * k), key);
+    unsigned long long* at = keys + i + (int64_t)g.n[0] * (j + (int64_t)g.n[1] * k);
+    const unsigned long long have = __ldcg(at);  // none yet: its distance is a NaN, which nothing exceeds
+    if (tri_farther(p, t, __uint_as_float((uint32_t)(have >> 32)))) return;
+    const float d2 = tri_d2_rn(p, t.a, t.b, t.c);
+    const unsigned long long key = ((unsigned long long)__float_as_uint(d2) << 32) | (uint32_t)t.id;
+    if (key >= have || !tri_box(p, g.hs, t.a, t.b, t.c)) return;
+    atomicMin(at, key);
 }
 
 constexpr int64_t kSmallPairs = 64;  // a thread tests a triangle's voxels itself up to this many
@@ -241,44 +251,47 @@ struct VoxPass {
     int32_t count;
 };
 
-// one thread per triangle and level: small ranges are tested here, large ones
-// listed (triangle, level) for k_df_vox_big
-__global__ void k_df_vox_small(const VoxPass vp, const Tris T, int2* big, unsigned* n_big)
+// One thread per triangle, level by level: small ranges are tested here, large
+// ones listed (leaf position, level) for k_df_vox_big; a full list leaves them
+// to the thread.
+__global__ void k_df_vox_small(const VoxPass vp, const Tris T, int2* big, unsigned* n_big, unsigned most_big)
 {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= T.n) return;
-    float A[3], B[3], C[3];
-    tri_verts(T, (int32_t)t, A, B, C);
+    const TriV v = tri_verts(T, (int32_t)t);
     for (int l = 0; l < vp.count; ++l) {
         const DfGrid& g = vp.g[l];
-        int64_t r0[3], r1[3];
-        if (!tri_range(g, A, B, C, r0, r1)) continue;
-        const int64_t count = (r1[0] - r0[0] + 1) * (r1[1] - r0[1] + 1) * (r1[2] - r0[2] + 1);
+        int32_t r0[3], r1[3];
+        if (!tri_range(g, v.a, v.b, v.c, r0, r1)) continue;
+        const int64_t count = (int64_t)(r1[0] - r0[0] + 1) * (r1[1] - r0[1] + 1) * (r1[2] - r0[2] + 1);
         if (count > kSmallPairs) {
-            big[atomicAdd(n_big, 1u)] = make_int2((int)t, l);
-            continue;
+            const unsigned at = atomicAdd(n_big, 1u);
+            if (at < most_big) {
+                big[at] = make_int2((int)t, l);
+                continue;
+            }
         }
-        for (int64_t k = r0[2]; k <= r1[2]; ++k)
-            for (int64_t j = r0[1]; j <= r1[1]; ++j)
-                for (int64_t i = r0[0]; i <= r1[0]; ++i) vox_pair(g, (int32_t)t, A, B, C, i, j, k, vp.keys[l]);
+        for (int32_t k = r0[2]; k <= r1[2]; ++k)
+            for (int32_t j = r0[1]; j <= r1[1]; ++j)
+                for (int32_t i = r0[0]; i <= r1[0]; ++i) vox_pair(g, v, i, j, k, vp.keys[l]);
     }
 }
 
 // one block per listed (triangle, level), threads over its voxels
-__global__ void k_df_vox_big(const VoxPass vp, const Tris T, const int2* big, const unsigned* n_big)
+__global__ void k_df_vox_big(const VoxPass vp, const Tris T, const int2* big, const unsigned* n_big, unsigned most_big)
 {
-    const unsigned nb = *n_big;
+    const unsigned nb = min(*n_big, most_big);
     for (unsigned b = blockIdx.x; b < nb; b += gridDim.x) {
         const int2 e = big[b];
         const DfGrid& g = vp.g[e.y];
-        float A[3], B[3], C[3];
-        tri_verts(T, e.x, A, B, C);
-        int64_t r0[3], r1[3];
-        tri_range(g, A, B, C, r0, r1);
+        const TriV v = tri_verts(T, e.x);
+        int32_t r0[3], r1[3];
+        tri_range(g, v.a, v.b, v.c, r0, r1);
         const int64_t sx = r1[0] - r0[0] + 1, sy = r1[1] - r0[1] + 1;
         const int64_t count = sx * sy * (r1[2] - r0[2] + 1);
         for (int64_t w = threadIdx.x; w < count; w += blockDim.x)
-            vox_pair(g, e.x, A, B, C, r0[0] + w % sx, r0[1] + (w / sx) % sy, r0[2] + w / (sx * sy), vp.keys[e.y]);
+            vox_pair(g, v, r0[0] + (int32_t)(w % sx), r0[1] + (int32_t)((w / sx) % sy), r0[2] + (int32_t)(w / (sx * sy)),
+                     vp.keys[e.y]);
     }
 }
 
@@ -288,6 +301,7 @@ __device__ __forceinline__ int64_t floordiv(int64_t x, int64_t y)  // y > 0
 }
 
 // sites from the voxelisation; on a cascade level also the coarser level's site
+// (an input index, like every site that a build leaves)
 __global__ void k_df_seed(const DfGrid g, const Tris T, const unsigned long long* keys, const int32_t* coarse,
                           const DfGrid gc, int32_t* sites)
 {
@@ -295,7 +309,6 @@ __global__ void k_df_seed(const DfGrid g, const Tris T, const unsigned long long
     if (s >= g.count) return;
     const unsigned long long key = keys[s];
     int32_t cur = key == ~0ull ? -1 : (int32_t)(key & 0xffffffffull);
-    float cd2 = __uint_as_float((uint32_t)(key >> 32));
     if (coarse) {
         const int64_t ii[3] = {s % g.n[0], (s / g.n[0]) % g.n[1], s / ((int64_t)g.n[0] * g.n[1])};
         int64_t jc[3];
@@ -304,54 +317,129 @@ __global__ void k_df_seed(const DfGrid g, const Tris T, const unsigned long long
             int64_t j = floordiv(g.ilo[a] + ii[a] + 1, 2) - gc.ilo[a];
             jc[a] = j < 0 ? 0 : (j > gc.n[a] - 1 ? gc.n[a] - 1 : j);
         }
-        float p[3];
-        df_pos(g, ii[0], ii[1], ii[2], p);
-        site_consider(T, p, coarse[jc[0] + (int64_t)gc.n[0] * (jc[1] + (int64_t)gc.n[1] * jc[2])], cur, cd2);
+        const int32_t t = coarse[jc[0] + (int64_t)gc.n[0] * (jc[1] + (int64_t)gc.n[1] * jc[2])];
+        if (t >= 0 && t != cur) {
+            float p[3];
+            df_pos(g, ii[0], ii[1], ii[2], p);
+            const TriV v = tri_verts(T, __ldg(T.slot + t));
+            if (site_better(tri_d2_rn(p, v.a, v.b, v.c), t, __uint_as_float((uint32_t)(key >> 32)), cur)) cur = t;
+        }
     }
-    sites[s] = cur;
+    sites[s] = cur < 0 ? -1 : __ldg(T.slot + cur);
 }
 
-// Neighbours mostly carry the same few sites: the distances of the last few
-// distinct candidates are kept, so each is evaluated once per sample.  The
-// result is the same minimum.
-constexpr int kSiteCache = 4;
+// One jump flooding step.  Triangles are small against the sample spacing, so the
+// 27 neighbours mostly carry different sites, few of which can be the best.  A
+// thread reads its neighbours' sites, all in flight together, takes its own
+// sample's site first, and lists the other distinct ones (a candidate equal to
+// one of the last kSiteCache listed is not listed again).  The warp then goes
+// through the lists: a candidate whose box is farther than the best so far is
+// done with; the (lane, candidate) pairs left are collected and evaluated 32 at a
+// time, the smaller (squared distance, input index) winning by a 64-bit minimum
+// in shared memory.  The result is the same minimum.
+// What bounds it is issue.  64^3 samples of the frame scene, us a step: 37 with
+// each candidate evaluated as it is met (once per neighbour for a few lanes at a
+// time), 30 with every listed one evaluated.
+constexpr int kSiteCache = 6;
+constexpr int kJfaBlock = 128;
 
-__global__ void k_df_jfa(const DfGrid g, const Tris T, const int32_t* in, int32_t* out, int32_t step)
+struct JfaShared {
+    float4 pos[32];
+    unsigned long long key[32];
+    int32_t site[64];  // collected pairs: the candidate ...
+    int32_t lane[64];  // ... and the lane whose sample it is for
+};
+
+__device__ __forceinline__ void jfa_pairs(const Tris& T, JfaShared& w, int first, int n)
 {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.count) return;
-    const int64_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int64_t i = s % nx, j = (s / nx) % ny, k = s / (nx * ny);
-    float p[3];
-    df_pos(g, i, j, k, p);
-    int32_t best = -1;
-    float bd2 = 0.f;
+    const int lane = (int)(threadIdx.x & 31u);
+    if (lane < n) {
+        const int to = w.lane[first + lane];
+        const TriV v = tri_verts(T, w.site[first + lane]);
+        const float4 q = w.pos[to];
+        const float p[3] = {q.x, q.y, q.z};
+        const float d2 = tri_d2_rn(p, v.a, v.b, v.c);
+        atomicMin(&w.key[to], (unsigned long long)__float_as_uint(d2) << 32 | (uint32_t)v.id);
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(kJfaBlock) k_df_jfa(const DfGrid g, const Tris T, const int32_t* __restrict__ in,
+                                                      int32_t* __restrict__ out, int32_t step)
+{
+    __shared__ int32_t list[26 * kJfaBlock];
+    __shared__ JfaShared shared[kJfaBlock / 32];
+    const unsigned full = 0xffffffffu;
+    JfaShared& w = shared[threadIdx.x / 32];
+    const int lane = (int)(threadIdx.x & 31u);
+    const int64_t s = (int64_t)blockIdx.x * kJfaBlock + threadIdx.x;
+    const bool on = s < g.count;
+    const int64_t s0 = on ? s : 0;
+    const int32_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const int32_t i = (int32_t)(s0 % nx), jk = (int32_t)(s0 / nx), j = jk % ny, k = jk / ny;
+    int32_t near[27];
+#pragma unroll
+    for (int q = 0; q < 27; ++q) {
+        const int64_t x = i + (int64_t)(q % 3 - 1) * step, y = j + (int64_t)(q / 3 % 3 - 1) * step, z = k + (int64_t)(q / 9 - 1) * step;
+        const bool inside = on && x >= 0 && x < nx && y >= 0 && y < ny && z >= 0 && z < nz;
+        near[q] = inside ? __ldg(in + x + nx * (y + (int64_t)ny * z)) : -1;
+    }
+    const int32_t own = near[13];
+    int listed = 0;
     int32_t seen[kSiteCache];
 #pragma unroll
     for (int c = 0; c < kSiteCache; ++c) seen[c] = -1;
-    for (int dz = -1; dz <= 1; ++dz) {
-        const int64_t z = k + dz * step;
-        if (z < 0 || z >= nz) continue;
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int64_t y = j + dy * step;
-            if (y < 0 || y >= ny) continue;
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int64_t x = i + dx * step;
-                if (x < 0 || x >= nx) continue;
-                const int32_t t = __ldg(in + x + nx * (y + ny * z));
-                if (t < 0) continue;
-                bool hit = false;
 #pragma unroll
-                for (int c = 0; c < kSiteCache; ++c) hit = hit || seen[c] == t;
-                if (hit) continue;  // already evaluated at this sample
+    for (int q = 0; q < 27; ++q) {
+        const int32_t t = near[q];
+        bool skip = t < 0 || t == own;
 #pragma unroll
-                for (int c = kSiteCache - 1; c > 0; --c) seen[c] = seen[c - 1];
-                seen[0] = t;
-                site_consider(T, p, t, best, bd2);
-            }
+        for (int c = 0; c < kSiteCache; ++c) skip = skip || seen[c] == t;
+        if (!skip) {
+#pragma unroll
+            for (int c = kSiteCache - 1; c > 0; --c) seen[c] = seen[c - 1];
+            seen[0] = t;
+            list[listed * kJfaBlock + threadIdx.x] = t;
+            ++listed;
         }
     }
-    out[s] = best;
+    float p[3];
+    df_pos(g, i, j, k, p);
+    w.pos[lane] = make_float4(p[0], p[1], p[2], 0.f);
+    unsigned long long key = ~0ull;
+    if (own >= 0) {
+        const TriV v = tri_verts(T, own);
+        key = (unsigned long long)__float_as_uint(tri_d2_rn(p, v.a, v.b, v.c)) << 32 | (uint32_t)v.id;
+    }
+    w.key[lane] = key;
+    __syncwarp();
+    const unsigned most = __reduce_max_sync(full, (unsigned)listed);
+    int pairs = 0;
+    for (unsigned c = 0; c < most; ++c) {
+        bool near_enough = false;
+        int32_t t = -1;
+        if (c < (unsigned)listed) {
+            t = list[c * kJfaBlock + threadIdx.x];
+            // no site yet: the key's distance is a NaN, which nothing exceeds
+            near_enough = !tri_farther(p, tri_verts(T, t), __uint_as_float((uint32_t)(w.key[lane] >> 32)));
+        }
+        const unsigned m = __ballot_sync(full, near_enough);
+        if (near_enough) {
+            const int at = pairs + __popc(m & ((1u << lane) - 1u));
+            w.site[at] = t;
+            w.lane[at] = lane;
+        }
+        pairs += __popc(m);
+        __syncwarp();
+        if (pairs >= 32) {
+            pairs -= 32;
+            jfa_pairs(T, w, pairs, 32);
+        }
+    }
+    if (pairs) jfa_pairs(T, w, 0, pairs);
+    if (!on) return;
+    key = w.key[lane];
+    out[s] = key == ~0ull ? -1 : __ldg(T.slot + (uint32_t)key);
 }
 
 // one thread per grid line along `axis`, walking in direction dir (+1 / -1).
@@ -405,131 +493,165 @@ __global__ void k_df_sweep(const SweepPass sp, const Tris T, int axis, int dir)
                 ii[ob] = ub;
                 float p[3];
                 df_pos(g, ii[0], ii[1], ii[2], p);
-                float cd2 = cur >= 0 ? site_d2(T, p, cur) : 0.f;
-                site_consider(T, p, prev, cur, cd2);
-                sites[base + q * stride[axis]] = cur;
+                const TriV pv = tri_verts(T, prev);
+                float cd2 = 0.f;
+                int32_t cid = -1;
+                if (cur >= 0) {
+                    const TriV cv = tri_verts(T, cur);
+                    cd2 = tri_d2_rn(p, cv.a, cv.b, cv.c);
+                    cid = cv.id;
+                }
+                if (site_better(tri_d2_rn(p, pv.a, pv.b, pv.c), pv.id, cd2, cid)) {
+                    cur = prev;
+                    sites[base + q * stride[axis]] = cur;
+                }
             }
             prev = cur;
         }
     }
 }
 
-// Both sweeps of one axis for one level: a thread takes one grid line, loads it
-// into shared memory, sweeps it in the + direction and then in the - direction
-// (lines of one axis are independent, so this equals all + sweeps followed by
-// all - sweeps), and writes it back.  The line is stored interleaved
-// (sample q of thread t at q * blockDim + t), so a warp's accesses to one q
-// fall in different banks.  The site carried along the line keeps its triangle
-// in registers: a step loads only the triangle of its own sample's site, and
-// only when the two sites differ.  Same operations, same order, same sites as
-// k_df_sweep.
+// Both sweeps of one axis for one level, one warp per grid line (lines of one
+// axis are independent, so the + sweep and then the - sweep of each line equal
+// all + sweeps followed by all - sweeps).
+//
+// Triangles are small against the sample spacing, so most samples of a line have
+// sites of their own and keep them.  A sample whose predecessor kept its site is
+// offered that site: this is known for all samples in advance, so the warp tests
+// 32 of them at a time.  Only where the offered site wins does the sweep go on in
+// sequence: the winner is carried to the next samples, again tested 32 at a time,
+// up to the first that keeps its own.  The triangles of the line's sites are read
+// once, into shared memory, and so is each sample's distance to its own site; a
+// sample holds the position of the sample its site came from.
+//
+// On a 64^3 level of the frame scene's cascade an axis took 50 to 210 us with one
+// thread per line (4,096 lines, under one warp per SM, about 1.6 us a step), and
+// 38 to 48 with the carried site tested ahead from every sample in turn.
 constexpr int kLineMax = 1024;  // longest line swept in shared memory
+constexpr int kLineBytes = 3 * 16 + 4 + 4;  // per sample: triangle (v0.w: input index), distance, site's origin
 
-// One step of a sweep at sample q.  CA/CB/CC hold the triangle of the sample's
-// own site `cur` (loaded one step ahead by the caller); PA/PB/PC the carried
-// site's, valid when prev_loaded.
-__device__ __forceinline__ void sweep_step(const DfGrid& g, const Tris& T, int64_t ii[3], int axis, int64_t q,
-                                           int32_t cur, const float CA[3], const float CB[3], const float CC[3],
-                                           int32_t& prev, float PA[3], float PB[3], float PC[3], bool& prev_loaded,
-                                           int32_t* slot)
+// the site that came from `carried` offered to sample q: whether it wins, and its distance there
+__device__ __forceinline__ bool line_offer(const DfGrid& g, int32_t ii[3], int axis, const float4* tri, const float* d2,
+                                           const int32_t* from, int q, int carried, float& d)
 {
-    if (prev >= 0 && prev != cur) {
-        ii[axis] = q;
-        float p[3];
-        df_pos(g, ii[0], ii[1], ii[2], p);
-        const float cd2 = cur >= 0 ? tri_d2_rn(p, CA, CB, CC) : 0.f;
-        if (!prev_loaded) {
-            tri_verts(T, prev, PA, PB, PC);
-            prev_loaded = true;
+    const int own = from[q];
+    const float4 a = tri[3 * carried], b = tri[3 * carried + 1], c = tri[3 * carried + 2];
+    const int32_t id = __float_as_int(a.w), own_id = own >= 0 ? __float_as_int(tri[3 * own].w) : -1;
+    if (own_id == id) return false;  // the same site: nothing changes
+    float p[3];
+    ii[axis] = q;
+    df_pos(g, ii[0], ii[1], ii[2], p);
+    const float va[3] = {a.x, a.y, a.z}, vb[3] = {b.x, b.y, b.z}, vc[3] = {c.x, c.y, c.z};
+    d = tri_d2_rn(p, va, vb, vc);
+    return site_better(d, id, d2[q], own_id);
+}
+
+__device__ __forceinline__ void sweep_line(const DfGrid& g, int32_t ii[3], int axis, const float4* tri, float* d2,
+                                           int32_t* from, int len, int dir)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = (int)(threadIdx.x & 31u);
+    auto at = [&](int step) { return dir > 0 ? step : len - 1 - step; };
+    int step = 1;
+    while (step < len) {
+        // the next 32 samples, each offered its predecessor's own site
+        const bool valid = step + lane < len;
+        const int q = valid ? at(step + lane) : 0;
+        const int before = valid ? from[at(step + lane - 1)] : -1;
+        float d = 0.f;
+        const bool wins = valid && before >= 0 && line_offer(g, ii, axis, tri, d2, from, q, before, d);
+        const unsigned m = __ballot_sync(full, wins);
+        if (m == 0u) {  // every one keeps its own
+            step += 32;
+            continue;
         }
-        const float d2 = tri_d2_rn(p, PA, PB, PC);
-        if (cur < 0 || d2 < cd2 || (d2 == cd2 && prev < cur)) {
-            cur = prev;  // the carried site wins and stays carried
-            *slot = cur;
-        } else {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {  // the sample's own site is carried on
-                PA[k] = CA[k];
-                PB[k] = CB[k];
-                PC[k] = CC[k];
+        const int first = __ffs(m) - 1;
+        const int carried = __shfl_sync(full, before, first);
+        if (lane == first) {
+            from[q] = carried;
+            d2[q] = d;
+        }
+        step += first + 1;
+        __syncwarp();
+        // the winner is carried on, up to the first sample that keeps its own site
+        // (one with the same site neither changes nor stops it)
+        while (step < len) {
+            const bool ok = step + lane < len;
+            const int r = ok ? at(step + lane) : 0;
+            float e = 0.f;
+            const bool takes = ok && line_offer(g, ii, axis, tri, d2, from, r, carried, e);
+            const bool same = ok && from[r] >= 0 && tri[3 * from[r]].w == tri[3 * carried].w;
+            const unsigned stop = __ballot_sync(full, ok && !takes && !same);
+            const int end = stop ? __ffs(stop) - 1 : 32;
+            __syncwarp();
+            if (takes && lane < end) {
+                from[r] = carried;
+                d2[r] = e;
             }
-        }
-    } else if (cur != prev) {
-        prev_loaded = false;  // a new carried site whose triangle is not loaded yet
-    }
-    prev = cur;
-}
-
-// the triangle of site t (nothing for t < 0)
-__device__ __forceinline__ void site_verts(const Tris& T, int32_t t, float A[3], float B[3], float C[3])
-{
-    if (t >= 0) tri_verts(T, t, A, B, C);
-}
-
-// one direction of a line's sweep: samples q0, q0 + dq, ... (len - 1 of them),
-// carrying from q0 - dq; the next sample's triangle is loaded a step ahead
-__device__ __forceinline__ void sweep_dir(const DfGrid& g, const Tris& T, int64_t ii[3], int axis, int32_t* L,
-                                          int64_t B, int64_t q0, int64_t dq, int64_t count)
-{
-    float PA[3], PB[3], PC[3], CA[3], CB[3], CC[3];
-    bool prev_loaded = false;
-    int32_t prev = L[(q0 - dq) * B];
-    int32_t cur = L[q0 * B];
-    site_verts(T, cur, CA, CB, CC);
-    for (int64_t k = 0; k < count; ++k) {
-        const int64_t q = q0 + k * dq;
-        int32_t nxt = -1;
-        float NA[3], NB[3], NC[3];
-        if (k + 1 < count) {
-            nxt = L[(q + dq) * B];
-            site_verts(T, nxt, NA, NB, NC);
-        }
-        sweep_step(g, T, ii, axis, q, cur, CA, CB, CC, prev, PA, PB, PC, prev_loaded, L + q * B);
-        cur = nxt;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            CA[c] = NA[c];
-            CB[c] = NB[c];
-            CC[c] = NC[c];
+            step += stop ? end + 1 : 32;
+            __syncwarp();
+            if (stop) break;
         }
     }
 }
 
 __global__ void k_df_sweep_line(const DfGrid g, const Tris T, int32_t* sites, int axis)
 {
-    extern __shared__ int32_t s_line[];
+    extern __shared__ float4 s_line[];
     const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
-    const int64_t n[3] = {g.n[0], g.n[1], g.n[2]};
-    const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (line >= n[oa] * n[ob]) return;
-    const int64_t stride[3] = {1, n[0], n[0] * n[1]};
-    int64_t ii[3];
-    ii[oa] = line % n[oa];
-    ii[ob] = line / n[oa];
-    ii[axis] = 0;
+    const int warps = (int)blockDim.x / 32, warp = (int)threadIdx.x / 32, lane = (int)(threadIdx.x & 31u);
+    const int64_t line = (int64_t)blockIdx.x * warps + warp;
+    if (line >= (int64_t)g.n[oa] * g.n[ob]) return;
+    const int len = g.n[axis];
+    float4* tri = s_line + (size_t)warp * 3 * len;
+    float* d2 = reinterpret_cast<float*>(s_line + (size_t)warps * 3 * len) + (size_t)warp * 2 * len;
+    int32_t* from = reinterpret_cast<int32_t*>(d2 + len);
+    const int64_t stride[3] = {1, g.n[0], (int64_t)g.n[0] * g.n[1]};
+    int32_t ii[3];
+    ii[oa] = (int32_t)(line % g.n[oa]);
+    ii[ob] = (int32_t)(line / g.n[oa]);
     const int64_t base = ii[oa] * stride[oa] + ii[ob] * stride[ob];
-    const int64_t len = n[axis];
-    const int64_t B = blockDim.x;
-    int32_t* L = s_line + threadIdx.x;
-    for (int64_t q = 0; q < len; ++q) L[q * B] = sites[base + q * stride[axis]];
-    sweep_dir(g, T, ii, axis, L, B, 1, 1, len - 1);         // + direction: samples 1 .. len-1
-    sweep_dir(g, T, ii, axis, L, B, len - 2, -1, len - 1);  // - direction: samples len-2 .. 0
-    for (int64_t q = 0; q < len; ++q) sites[base + q * stride[axis]] = L[q * B];
+    for (int q = lane; q < len; q += 32) {
+        const int32_t k = sites[base + q * stride[axis]];
+        from[q] = k >= 0 ? q : -1;
+        d2[q] = 0.f;
+        if (k >= 0) {
+            const float4* v = T.tris + 3 * (int64_t)k;
+            const float4 a = __ldg(v), b = __ldg(v + 1), c = __ldg(v + 2);
+            tri[3 * q] = a;
+            tri[3 * q + 1] = make_float4(b.x, b.y, b.z, __int_as_float(k));  // v1.w: leaf position
+            tri[3 * q + 2] = c;
+            float p[3];
+            ii[axis] = q;
+            df_pos(g, ii[0], ii[1], ii[2], p);
+            const float va[3] = {a.x, a.y, a.z}, vb[3] = {b.x, b.y, b.z}, vc[3] = {c.x, c.y, c.z};
+            d2[q] = tri_d2_rn(p, va, vb, vc);
+        }
+    }
+    __syncwarp();
+    sweep_line(g, ii, axis, tri, d2, from, len, 1);
+    sweep_line(g, ii, axis, tri, d2, from, len, -1);
+    for (int q = lane; q < len; q += 32) {
+        const int o = from[q];
+        if (o != q && o >= 0) sites[base + q * stride[axis]] = __float_as_int(tri[3 * o + 1].w);
+    }
 }
 
-// signed distance to the site triangle (the exact bake's closest point and sign)
-__global__ void k_df_field(const DfGrid g, const Tris T, const float4* pn, const int32_t* sites, void* grid,
-                           int32_t f16)
+// The end of a level: its sites as input indices, and (grid non-null) the signed
+// distance to each site's triangle (the exact bake's closest point and sign).
+__global__ void k_df_finish(const DfGrid g, const Tris T, const float4* pn, const int32_t* sites, int32_t* ids, void* grid,
+                            int32_t f16)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= g.count) return;
-    const int32_t t = sites[s];
+    const int32_t k = sites[s];
+    ids[s] = k >= 0 ? __float_as_int(__ldg(&T.tris[3 * (int64_t)k].w)) : -1;
+    if (!grid) return;
     float v = __int_as_float(0x7f800000);
-    if (t >= 0) {
+    if (k >= 0) {
         float pp[3];
         df_pos(g, s % g.n[0], (s / g.n[0]) % g.n[1], s / ((int64_t)g.n[0] * g.n[1]), pp);
         const float3 p = make_float3(pp[0], pp[1], pp[2]);
-        const int32_t k = __ldg(T.slot + t);
         rtbake::Nearest nb = {__int_as_float(0x7f800000), -1, 0x7fffffff};
         rtbake::consider(nb, p, T.tris, k);
         v = rtbake::signed_distance(p, nb, T.tris, pn);
@@ -577,39 +699,38 @@ DfGrid df_grid(const rt_sdf* sdf, int k)
 
 unsigned blocks_for(int64_t n) { return (unsigned)((n + kBlock - 1) / kBlock); }
 
+constexpr int64_t kBigMost = 1 << 18;  // large (triangle, level) pairs listed for a block each
+
 // Steps 1..stage for the levels `lv[0..nl)` (0 for a single grid), given in
 // the order they are built (coarsest first).  All levels are voxelised in one
 // pass over the triangles (a level's voxel candidates do not depend on the
 // other levels); then each level in turn is seeded (on a cascade also from the
-// next coarser level's finished sites in `jfa`), flooded and swept, leaving its
-// sites in `jfa` before the next finer level reads them.  The sites of every
-// listed level also go to `out`.  jfa, out: one int32 per sample of every
-// level (indexed by level), device.
-rt_status df_build(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t stage, int32_t* jfa,
-                   int32_t* out, cudaStream_t s)
+// next coarser level's finished sites in `ids`), flooded and swept, leaving its
+// sites in `ids` (one input index per sample of every level, device) before the
+// next finer level reads them, and with `values` its field values in the grid.
+rt_status df_build(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t stage, int32_t* ids, bool values,
+                   cudaStream_t s)
 {
     const Tris T = {sc->tris, sc->slot, sc->n_tris};
     const int64_t per = (int64_t)sdf->n[0] * sdf->n[1] * sdf->n[2];
     if (per > 0x7fffffffLL * (int64_t)kBlock) return rt_fail(RT_ERR_INVALID_ARG, "grid too large");
     const int cascade_levels = sdf->levels;
 
-    // scratch: keys of every listed level, one spare site buffer, the large-triangle list
-    const size_t keys_bytes = (size_t)per * 8 * nl, tmp_bytes = (size_t)per * 4, big_bytes = (size_t)T.n * 8 * nl;
-    const size_t total = keys_bytes + tmp_bytes + big_bytes + 4 * 256;
-    char* base = nullptr;
-    RT_CUDA_TRY(cudaMallocAsync((void**)&base, total, s));
+    // scratch: keys of every listed level, two site buffers, the large-triangle list
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    size_t off = 0;
-    unsigned long long* keys = reinterpret_cast<unsigned long long*>(base + off);
-    off = align(off + keys_bytes);
-    int32_t* tmp = reinterpret_cast<int32_t*>(base + off);
-    off = align(off + tmp_bytes);
-    int2* big = reinterpret_cast<int2*>(base + off);
-    off = align(off + big_bytes);
-    unsigned* n_big = reinterpret_cast<unsigned*>(base + off);
+    const unsigned most_big = (unsigned)(T.n * nl < kBigMost ? T.n * nl : kBigMost);
+    const size_t keys_bytes = align((size_t)per * 8 * nl), sites_bytes = align((size_t)per * 4);
+    const size_t big_bytes = align((size_t)most_big * sizeof(int2));
+    void* scratch = nullptr;
+    rt_status st = rt_scratch_alloc(&scratch, keys_bytes + 2 * sites_bytes + big_bytes + 256, s);
+    if (st != RT_OK) return st;
+    char* base = static_cast<char*>(scratch);
+    unsigned long long* keys = reinterpret_cast<unsigned long long*>(base);
+    int32_t* work[2] = {reinterpret_cast<int32_t*>(base + keys_bytes), reinterpret_cast<int32_t*>(base + keys_bytes + sites_bytes)};
+    int2* big = reinterpret_cast<int2*>(base + keys_bytes + 2 * sites_bytes);
+    unsigned* n_big = reinterpret_cast<unsigned*>(base + keys_bytes + 2 * sites_bytes + big_bytes);
 
-    rt_status st = RT_OK;
-    cudaError_t e = cudaMemsetAsync(keys, 0xff, keys_bytes, s);
+    cudaError_t e = cudaMemsetAsync(keys, 0xff, (size_t)per * 8 * nl, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(n_big, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) st = rt_cuda_fail(e, "cudaMemsetAsync");
 
@@ -625,57 +746,51 @@ rt_status df_build(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl,
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        k_df_vox_small<<<blocks_for(T.n), kBlock, 0, s>>>(vp, T, big, n_big);
-        k_df_vox_big<<<(unsigned)(sms > 0 ? sms * 4 : 512), kBlock, 0, s>>>(vp, T, big, n_big);
+        k_df_vox_small<<<blocks_for(T.n), kBlock, 0, s>>>(vp, T, big, n_big, most_big);
+        k_df_vox_big<<<(unsigned)(sms > 0 ? sms * 4 : 512), kBlock, 0, s>>>(vp, T, big, n_big, most_big);
     }
     // 2.-3. per level, coarsest first: seeding, jump flooding, the six sweeps
+    const int64_t esz = sdf->dtype == RT_GRID_F16 ? 2 : 4;
     for (int l = 0; l < nl && st == RT_OK; ++l) {
         const int k = lv[l];
-        int32_t* sites = jfa + (int64_t)k * per;
         const DfGrid g = df_grid(sdf, k);
         DfGrid gc;
         memset(&gc, 0, sizeof(gc));
         const int32_t* coarse = nullptr;
         if (cascade_levels > 0 && k + 1 < cascade_levels) {
             gc = df_grid(sdf, k + 1);
-            coarse = jfa + (int64_t)(k + 1) * per;
+            coarse = ids + (int64_t)(k + 1) * per;
         }
+        int32_t* sites = work[0];
+        int32_t* other = work[1];
         k_df_seed<<<blocks_for(g.count), kBlock, 0, s>>>(g, T, keys + (size_t)l * per, coarse, gc, sites);
         if (stage >= 2) {
             int64_t nmax = g.n[0] > g.n[1] ? g.n[0] : g.n[1];
             if (g.n[2] > nmax) nmax = g.n[2];
             int64_t step = 1;
             while (2 * step < nmax) step *= 2;
-            int32_t* a = sites;
-            int32_t* b = tmp;
             for (; step >= 1; step /= 2) {
-                k_df_jfa<<<blocks_for(g.count), kBlock, 0, s>>>(g, T, a, b, (int32_t)step);
-                int32_t* t = a;
-                a = b;
-                b = t;
-            }
-            if (a != sites) {
-                e = cudaMemcpyAsync(sites, a, (size_t)g.count * 4, cudaMemcpyDeviceToDevice, s);
-                if (e != cudaSuccess) st = rt_cuda_fail(e, "cudaMemcpyAsync");
+                k_df_jfa<<<(unsigned)((g.count + kJfaBlock - 1) / kJfaBlock), kJfaBlock, 0, s>>>(g, T, sites, other, (int32_t)step);
+                int32_t* t = sites;
+                sites = other;
+                other = t;
             }
         }
-        if (st == RT_OK && stage >= 3) {
-            for (int axis = 0; axis < 3; ++axis) {
+        if (stage >= 3) {
+            for (int axis = 0; axis < 3 && st == RT_OK; ++axis) {
                 const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
                 const int64_t lines = (int64_t)g.n[oa] * g.n[ob];
                 if (g.n[axis] <= kLineMax) {
-                    const int threads = g.n[axis] <= 512 ? 64 : 32;
-                    const size_t smem = (size_t)threads * g.n[axis] * sizeof(int32_t);
+                    // four lines a block while they fit in 48 KB of shared memory
+                    const size_t line_bytes = (size_t)g.n[axis] * kLineBytes;
+                    const int warps = 4 * line_bytes <= (48 << 10) ? 4 : (2 * line_bytes <= (48 << 10) ? 2 : 1);
+                    const size_t smem = warps * line_bytes;
                     if (smem > 48 * 1024) {
-                        e = cudaFuncSetAttribute(k_df_sweep_line, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem);
-                        if (e != cudaSuccess) {
-                            st = rt_cuda_fail(e, "cudaFuncSetAttribute");
-                            break;
-                        }
+                        e = cudaFuncSetAttribute(k_df_sweep_line, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                        if (e != cudaSuccess) st = rt_cuda_fail(e, "cudaFuncSetAttribute");
                     }
-                    k_df_sweep_line<<<(unsigned)((lines + threads - 1) / threads), threads, smem, s>>>(g, T, sites,
-                                                                                                      axis);
+                    if (st == RT_OK)
+                        k_df_sweep_line<<<(unsigned)((lines + warps - 1) / warps), 32 * warps, smem, s>>>(g, T, sites, axis);
                 } else {
                     SweepPass sp;
                     memset(&sp, 0, sizeof(sp));
@@ -688,35 +803,18 @@ rt_status df_build(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl,
                 }
             }
         }
-        if (st == RT_OK && out != jfa) {
-            e = cudaMemcpyAsync(out + (int64_t)k * per, sites, (size_t)g.count * 4, cudaMemcpyDeviceToDevice, s);
-            if (e != cudaSuccess) st = rt_cuda_fail(e, "cudaMemcpyAsync");
-        }
+        void* grid = values ? static_cast<char*>(const_cast<void*>(sdf->grid)) + k * per * esz : nullptr;
+        if (st == RT_OK)
+            k_df_finish<<<blocks_for(g.count), kBlock, 0, s>>>(g, T, sc->pn, sites, ids + (int64_t)k * per, grid,
+                                                               sdf->dtype == RT_GRID_F16);
     }
     if (st == RT_OK) {
         e = cudaGetLastError();
         if (e != cudaSuccess) st = rt_cuda_fail(e, "field build launch");
     }
-    e = cudaFreeAsync(base, s);
+    e = cudaFreeAsync(scratch, s);
     if (st == RT_OK && e != cudaSuccess) st = rt_cuda_fail(e, "cudaFreeAsync");
     return st;
-}
-
-rt_status field_values(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, const int32_t* sites,
-                       cudaStream_t s)
-{
-    const Tris T = {sc->tris, sc->slot, sc->n_tris};
-    const int64_t per = (int64_t)sdf->n[0] * sdf->n[1] * sdf->n[2];
-    const int64_t esz = sdf->dtype == RT_GRID_F16 ? 2 : 4;
-    for (int l = 0; l < nl; ++l) {
-        const int k = lv[l];
-        const DfGrid g = df_grid(sdf, k);
-        char* grid = static_cast<char*>(const_cast<void*>(sdf->grid)) + k * per * esz;
-        k_df_field<<<blocks_for(g.count), kBlock, 0, s>>>(g, T, sc->pn, sites + k * per, grid,
-                                                        sdf->dtype == RT_GRID_F16);
-    }
-    RT_CUDA_TRY(cudaGetLastError());
-    return RT_OK;
 }
 
 }  // namespace
@@ -730,29 +828,14 @@ rt_status rt_launch_df_sites(const rt_scene* sc, const rt_sdf* sdf, int32_t stag
     int lv[RT_MAX_LEVELS];
     const int nl = sdf->levels > 0 ? sdf->levels : 1;
     for (int l = 0; l < nl; ++l) lv[l] = nl - 1 - l;  // coarsest first
-    const int64_t count = (int64_t)nl * sdf->n[0] * sdf->n[1] * sdf->n[2];
-    int32_t* jfa = nullptr;
-    RT_CUDA_TRY(cudaMallocAsync((void**)&jfa, (size_t)count * 4, s));
-    rt_status st = df_build(sc, sdf, lv, nl, stage, jfa, d_sites, s);
-    cudaError_t e = cudaFreeAsync(jfa, s);
-    if (st == RT_OK && e != cudaSuccess) st = rt_cuda_fail(e, "cudaFreeAsync");
-    return st;
+    return df_build(sc, sdf, lv, nl, stage, d_sites, false, s);
 }
 
 // The listed levels (all of them for a full build; the moved ones of a rolling
-// update), coarsest first: finished sites into `jfa_store` (kept by the
-// handle: the seeds of finer levels later), field values from them.
-rt_status rt_launch_df_levels(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t* jfa_store,
-                              cudaStream_t s)
+// update), coarsest first: finished sites into `ids` (kept by the handle: the
+// seeds of finer levels later), field values from them.
+rt_status rt_launch_df_levels(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t* ids, cudaStream_t s)
 {
     if (nl <= 0) return RT_OK;
-    const int levels = sdf->levels > 0 ? sdf->levels : 1;
-    const int64_t count = (int64_t)levels * sdf->n[0] * sdf->n[1] * sdf->n[2];
-    int32_t* out = nullptr;
-    RT_CUDA_TRY(cudaMallocAsync((void**)&out, (size_t)count * 4, s));
-    rt_status st = df_build(sc, sdf, lv, nl, 3, jfa_store, out, s);
-    if (st == RT_OK) st = field_values(sc, sdf, lv, nl, out, s);
-    cudaError_t e = cudaFreeAsync(out, s);
-    if (st == RT_OK && e != cudaSuccess) st = rt_cuda_fail(e, "cudaFreeAsync");
-    return st;
+    return df_build(sc, sdf, lv, nl, 3, ids, true, s);
 }
