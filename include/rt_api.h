@@ -170,15 +170,15 @@ rt_status rt_sdf_create(const void* d_grid, int32_t dtype, const float lo[3], co
                         const int32_t n[3], rt_sdf** out);
 rt_status rt_sdf_destroy(rt_sdf* sdf);
 
-/* Build (or rebuild) the library's cell-corner copy of the grid of `sdf`:
- * for every cell the 8 corner values stored together (32 bytes for float32,
- * 16 bytes for float16), so that a march step reads one vector instead of 8
- * scalars.  Same values, same arithmetic, same results.  rt_sdf_bake calls it
+/* Build (or rebuild) the library's cell copy of the grid of `sdf`: for every
+ * cell face across x its 4 corner values stored together (16 bytes for float32,
+ * 8 bytes for float16), so that a march step reads two adjacent vectors instead
+ * of 8 scalars.  Same values, same arithmetic, same results.  rt_sdf_bake calls it
  * itself; call it after writing the grid memory any other way (for example
  * after an optimiser step), otherwise the traces keep reading the old copy.
  * Traces read the plain grid until the first prepare, or when the tuning
  * selects the plain layout.  Also builds the x-pair copy (see rt_tuning).
- * Memory: about 8x (cells) + 2x (pairs) the grid, owned by the handle,
+ * Memory: about 4x (cells) + 2x (pairs) the grid, owned by the handle,
  * released by rt_sdf_destroy.  On a cascade: the cell copy of every level
  * (no x-pair copy).  Enqueued on `stream`. */
 rt_status rt_sdf_prepare(rt_sdf* sdf, void* stream);
@@ -266,7 +266,7 @@ rt_status rt_cascade_create(const void* d_grid, int32_t dtype, int32_t levels, i
  * method); a level that moved by n or more samples on an axis is baked
  * whole.  After an RT_BAKE_JFA bake, each moved level is rebuilt whole by the
  * paper's build instead, seeded from the next coarser level's sites.  The
- * cell-corner copy of each changed level is rebuilt.  The values equal those
+ * cell copy of each changed level is rebuilt.  The values equal those
  * of a full rt_sdf_bake at the new centre (with the same method).  Enqueued on
  * `stream`; uses a device scratch of one level owned by the handle (allocated
  * on the first call).  *moved (nullable) receives the number of levels that
@@ -445,7 +445,7 @@ rt_status rt_trace_combined_backward(const rt_scene* scene, const rt_sdf* sdf, c
  *                 compressed tree (80-byte nodes, 8-bit child bounds,
  *                 octant-ordered children).  Scenes whose wide tree would be
  *                 deeper than its traversal stack use the binary tree.
- *   grid_layout   RT_LAYOUT_CELLS (default): use the cell-corner copy when it
+ *   grid_layout   RT_LAYOUT_CELLS (default): use the cell copy when it
  *                 exists; RT_LAYOUT_PLAIN: always read the plain grid;
  *                 RT_LAYOUT_PAIRS: the copy of x-neighbour pairs (4 loads a
  *                 step, twice the grid's size) when it exists

@@ -295,7 +295,7 @@ def rt_sdf_bake(scene: Scene, sdf: Sdf, method: int = BAKE_AUTO, stream=None) ->
 
 
 def rt_sdf_prepare(sdf: Sdf, stream=None) -> None:
-    """(Re)build the cell-corner copy of the grid; call after writing the grid tensor."""
+    """(Re)build the cell copy of the grid; call after writing the grid tensor."""
     _check(lib().rt_sdf_prepare(sdf.handle, _stream(stream)))
 
 

@@ -2,7 +2,7 @@
 
 The candidates cover the knobs of rt_set_tuning: kernel (wavefront stages with
 per-lane refill, or one thread per query), threads per block, resident blocks
-per SM, the refill threshold, the grid layout (cell-corner copy or plain
+per SM, the refill threshold, the grid layout (cell copy or plain
 grid), the tree width, and the query order (bits of the origin lattice, or
 none).  Results never depend on the tuning, only the time does.
 """

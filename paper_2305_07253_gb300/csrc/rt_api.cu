@@ -405,12 +405,12 @@ extern "C" rt_status rt_cascade_recenter(const rt_scene* sc, rt_sdf* sdf, const 
         }
         st = rt_launch_cascade_bake(sc, sdf, k, keep, shift, s);
         if (st != RT_OK) return st;
-        st = rt_launch_cascade_cells(sdf, k, s);
+        st = rt_launch_cascade_cells(sdf, k, 1, s);
         if (st != RT_OK) return st;
     }
     if (n_rebuilt > 0) {
         st = rt_launch_df_levels(sc, sdf, rebuilt, n_rebuilt, sdf->sites, s);
-        for (int l = 0; l < n_rebuilt && st == RT_OK; ++l) st = rt_launch_cascade_cells(sdf, rebuilt[l], s);
+        for (int l = 0; l < n_rebuilt && st == RT_OK; ++l) st = rt_launch_cascade_cells(sdf, rebuilt[l], 1, s);
         if (st != RT_OK) return st;
     }
     float lo[3], hi[3], h, ih;

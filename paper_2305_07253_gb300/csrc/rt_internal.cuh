@@ -22,10 +22,10 @@
 //            plane test (inf: a badly shaped triangle, never decided by its plane)
 //   slot   : 4 B per triangle: input index -> leaf-order position (field build)
 //   grid   : caller memory, dense n0*n1*n2 float32 or float16, x fastest
-//   cells  : optional library copy of the grid with the 8 corners of every cell
-//            stored together (32 B float32 / 16 B float16 per cell, cells x
-//            fastest), so one march step is one vector load instead of eight
-//            scalar ones; identical values, identical arithmetic
+//   cells  : optional library copy of the grid with the four values of every cell
+//            face across x stored together (16 B float32 / 8 B float16 per entry,
+//            x fastest), so one march step is two adjacent vector loads instead
+//            of eight scalar ones; identical values, identical arithmetic
 //   pairs  : optional library copy with the two x-neighbours (i, i+1) of every
 //            sample stored together (8 B float32 / 4 B float16, (n0-1) x n1 x n2,
 //            x fastest): a march step is four small loads from a copy twice the
@@ -75,13 +75,13 @@ struct rt_sdf {
     int32_t dtype;
     float lo[3], hi[3], h[3], ih[3];  // one grid; on a cascade: the coarsest level's box
     int32_t n[3];
-    void* cells;        // library-owned cell-corner copy (null until rt_sdf_prepare)
+    void* cells;        // library-owned cell copy (null until rt_sdf_prepare)
     int64_t cells_bytes;
     void* pairs;        // library-owned x-pair copy (null until rt_sdf_prepare)
     int64_t pairs_bytes;
     int device;
     // cascade (levels > 0): level k holds n^3 samples at (ilo[k] + i) * h0 * 2^k,
-    // stored at grid + k * n^3, its cells at cells + k * (n-1)^3
+    // stored at grid + k * n^3, its cells at cells + k * n (n-1)^2 entries
     int32_t levels;
     float h0;
     int32_t ilo[RT_MAX_LEVELS][3];
@@ -138,7 +138,7 @@ struct TraceArgs {
     int32_t mode, any_hit, refine_root;
     float m_near, m_far;
     int32_t levels;        // 0: one grid; > 0: a cascade read through its cell copy
-    int64_t level_cells;   // cells per cascade level
+    int64_t level_cells;   // entries of the cell copy per cascade level
     CascLevel lv[RT_MAX_LEVELS];
     const float4* rays;
     rt_hit* hits;
@@ -266,6 +266,6 @@ rt_status rt_fill_trace_args(TraceArgs& a, const rt_scene* sc, const rt_sdf* sdf
 void rt_cascade_geometry(const rt_sdf* sdf, int k, float lo[3], float hi[3], float* h, float* ih);
 rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, const void* keep, const int32_t shift[3],
                                  cudaStream_t s);
-rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int k, cudaStream_t s);
+rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int first, int count, cudaStream_t s);
 rt_status rt_launch_df_sites(const rt_scene* sc, const rt_sdf* sdf, int32_t stage, int32_t* d_sites, cudaStream_t s);
 rt_status rt_launch_df_levels(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl, int32_t* ids, cudaStream_t s);

@@ -440,7 +440,7 @@ __device__ __forceinline__ bool bvh_segment(const TraceArgs& a, float3 o, float3
 // ---------------------------------------------------------------------------
 // Grid storage seen by the march, fixed at compile time so that a step has no
 // layout or type branches: the caller's plain grid (float32 / float16) or the
-// library's cell-corner copy (float32 / float16).
+// library's cell copy (float32 / float16).
 enum GridLayout { GL_PLAIN_F32 = 0, GL_PLAIN_F16 = 1, GL_CELLS_F32 = 2, GL_CELLS_F16 = 3, GL_PAIRS_F32 = 4,
                   GL_PAIRS_F16 = 5, GL_CASC_F32 = 6, GL_CASC_F16 = 7 };
 
@@ -488,19 +488,54 @@ __device__ __forceinline__ int64_t grid_base(const TraceArgs& a, const Cell& c)
     return c.i0[0] + (int64_t)a.gn[0] * (c.i0[1] + (int64_t)a.gn[1] * c.i0[2]);
 }
 
-// Position of cell (i, j, k) in the cell copy, x fastest.  Orders that keep
-// 3-d neighbours in one 128-byte line were measured on the 1080p GI workload,
-// records unchanged: 2x2 blocks in x-y 0.743 ms, 2x2x2 blocks 0.750 ms,
-// against 0.739 ms; a 4x4x4 brick order 0.855 against 0.837 ms (earlier kernel).
+// The cell copy: entry (i, j, k), i < nx, j < ny-1, k < nz-1, x fastest, holds the
+// four values (i, j, k), (i, j+1, k), (i, j, k+1), (i, j+1, k+1); a cell is entry i
+// and the next one, two adjacent loads.  A march waits on its cell loads, and the
+// copy's size decides how many of them miss the L2: with all eight corners in
+// each entry (twice the bytes, one load) the field-only call took 0.490 ms against
+// 0.447 on 2,073,600 GI rays at 256^3 (531 against 268 MB), and a shadow call
+// 0.490 against 0.469.  On a cascade, whose copy fits the L2 either way, there is
+// no difference.  Orders of the eight-corner cells that keep 3-d neighbours in one
+// 128-byte line were no faster: 2x2 blocks in x-y 0.743 ms, 2x2x2 blocks 0.750 ms,
+// against 0.739 ms (combined call, an earlier kernel).
 __host__ __device__ __forceinline__ int64_t cell_slot(int i, int j, int k, int nx, int ny)
 {
-    return i + (int64_t)(nx - 1) * (j + (int64_t)(ny - 1) * k);
+    return i + (int64_t)nx * (j + (int64_t)(ny - 1) * k);
 }
 
-// cells the copy of an nx x ny x nz grid holds
+// entries the copy of an nx x ny x nz grid holds
 __host__ __device__ __forceinline__ int64_t cell_count(int nx, int ny, int nz)
 {
-    return (int64_t)(nx - 1) * (ny - 1) * (nz - 1);
+    return (int64_t)nx * (ny - 1) * (nz - 1);
+}
+
+// the 8 corner values of the cell at entry idx of the copy, order
+// v000 v100 v010 v110 v001 v101 v011 v111
+template <bool F16>
+__device__ __forceinline__ void load_cell(const void* cells, int64_t idx, float v[8])
+{
+    if (F16) {
+        const uint2* q = reinterpret_cast<const uint2*>(cells) + idx;
+        const uint2 e[2] = {__ldg(q), __ldg(q + 1)};
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            const __half2 lo = *reinterpret_cast<const __half2*>(&e[x].x), hi = *reinterpret_cast<const __half2*>(&e[x].y);
+            v[x] = __low2float(lo);
+            v[2 + x] = __high2float(lo);
+            v[4 + x] = __low2float(hi);
+            v[6 + x] = __high2float(hi);
+        }
+    } else {
+        const float4* q = reinterpret_cast<const float4*>(cells) + idx;
+        const float4 e[2] = {__ldg(q), __ldg(q + 1)};
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            v[x] = e[x].x;
+            v[2 + x] = e[x].y;
+            v[4 + x] = e[x].z;
+            v[6 + x] = e[x].w;
+        }
+    }
 }
 
 __device__ __forceinline__ int64_t cell_index(const TraceArgs& a, const Cell& c)
@@ -512,19 +547,8 @@ __device__ __forceinline__ int64_t cell_index(const TraceArgs& a, const Cell& c)
 template <int L>
 __device__ __forceinline__ void corners(const TraceArgs& a, const Cell& c, float v[8])
 {
-    if (L == GL_CELLS_F16) {
-        uint4 q = __ldg(reinterpret_cast<const uint4*>(a.cells) + cell_index(a, c));
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            __half2 h2 = *reinterpret_cast<const __half2*>(&w[k]);
-            v[2 * k] = __low2float(h2);
-            v[2 * k + 1] = __high2float(h2);
-        }
-        return;
-    }
-    if (L == GL_CELLS_F32) {
-        ldg8(reinterpret_cast<const float*>(a.cells) + 8 * cell_index(a, c), v);
+    if (L == GL_CELLS_F16 || L == GL_CELLS_F32) {
+        load_cell<L == GL_CELLS_F16>(a.cells, cell_index(a, c), v);
         return;
     }
     if (L == GL_PAIRS_F32 || L == GL_PAIRS_F16) {
@@ -570,18 +594,6 @@ __device__ __forceinline__ float interp8(const float f[3], const float v[8])
     float c0 = lerp_rn(f[1], c00, c10);
     float c1 = lerp_rn(f[1], c01, c11);
     return lerp_rn(f[2], c0, c1);
-}
-
-// the 8 corners of a 16-byte half-precision cell, held as 4 words in v[0..3], widened in place
-__device__ __forceinline__ void widen_f16_cell(float v[8])
-{
-    const uint32_t w[4] = {__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3])};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        __half2 h2 = *reinterpret_cast<const __half2*>(&w[k]);
-        v[2 * k] = __low2float(h2);
-        v[2 * k + 1] = __high2float(h2);
-    }
 }
 
 template <int L>
@@ -634,16 +646,7 @@ __device__ __forceinline__ float casc_trilinear(const TraceArgs& a, int k, float
     float f[3];
     const int64_t idx = casc_locate(a, k, px, py, pz, f);
     float v[8];
-    if (L == GL_CASC_F16) {
-        uint4 q = __ldg(reinterpret_cast<const uint4*>(a.cells) + idx);
-        v[0] = __uint_as_float(q.x);
-        v[1] = __uint_as_float(q.y);
-        v[2] = __uint_as_float(q.z);
-        v[3] = __uint_as_float(q.w);
-        widen_f16_cell(v);
-    } else {
-        ldg8(reinterpret_cast<const float*>(a.cells) + 8 * idx, v);
-    }
+    load_cell<L == GL_CASC_F16>(a.cells, idx, v);
     return interp8(f, v);
 }
 
@@ -725,7 +728,9 @@ __device__ __forceinline__ March sdf_march(const TraceArgs& a, float3 o, float3 
     return m;
 }
 
-// root of phi(o + s d) = eps_hit inside the last step [t_prev, t] (24 halvings)
+// Root of phi(o + s d) = eps_hit inside the last step [t_prev, t] (24 halvings).
+// phi >= eps_hit at t_prev and phi < eps_hit at t: once the middle is one of the
+// ends, further halvings change nothing.
 template <int L>
 __device__ __forceinline__ float refine(const TraceArgs& a, float3 o, float3 d, float t_prev, float t)
 {
@@ -735,7 +740,9 @@ __device__ __forceinline__ float refine(const TraceArgs& a, float3 o, float3 d, 
         float eps_hit, eps_min;
         float phi = field_at<L>(a, __fmaf_rn(mid, d.x, o.x), __fmaf_rn(mid, d.y, o.y), __fmaf_rn(mid, d.z, o.z),
                                 eps_hit, eps_min);
+        const bool ended = mid == lo || mid == hi;
         if (phi < eps_hit) hi = mid; else lo = mid;
+        if (ended) break;
     }
     return 0.5f * (lo + hi);
 }
