@@ -416,9 +416,10 @@ rt_status rt_trace_batches(const rt_scene* scene, const rt_sdf* sdf, const rt_ba
  * with w_k the 8 trilinear weights.  Adds d_grad_t[i] * dt/dtheta_k into
  * d_grad_grid[k] (float32, same layout as the grid; the caller zeroes it).
  * Queries with grad phi . d > -1e-6 (tangent), a field hit at the start of
- * the sub-interval, or another tracer contribute nothing.  The forward pass
- * is not stored: the kernel re-marches each ray.  The grid must be
- * RT_GRID_F32 and not a cascade. */
+ * the sub-interval, or another tracer contribute nothing.  The root is the
+ * record's t; a record whose t is not a root of this grid's phi (it came from a
+ * call without refine_root, or the grid has changed since) is marched again.
+ * The grid must be RT_GRID_F32 and not a cascade. */
 rt_status rt_trace_combined_backward(const rt_scene* scene, const rt_sdf* sdf, const rt_ray* d_rays,
                                      int64_t n, const rt_split_params* params, const rt_hit* d_hits,
                                      const float* d_grad_t, float* d_grad_grid, void* stream);
