@@ -5,7 +5,7 @@
 // (phi = sum_k w_k(p) theta_k with the trilinear weights w_k), so implicit
 // differentiation gives dt/dtheta_k = -w_k(p*) / (grad phi(p*) . d).  The root is
 // the record's t (a forward call with refine_root); a record whose t is not one
-// (phi there is not eps_hit to rounding: a forward call without refine_root, or
+// (phi does not cross eps_hit there: a forward call without refine_root, or
 // another grid since) is marched again with the forward code (same roundings,
 // same steps) and its root refined in the last step.  grad_t * dt/dtheta_k is
 // scattered into the gradient grid.
@@ -37,12 +37,17 @@ __global__ void __launch_bounds__(kBwdBlock) k_backward(const TraceArgs a, const
         ts = s.t1;
         te = s.t2;
     }
-    float t = a.hits[i].t, e0, e1;
-    // A root: phi within a few ulp of eps_hit, over the ulp of t that separates the
-    // refined bracket's ends and those of the position and of phi's corners.
-    const float phi = field_at<L>(a, __fmaf_rn(t, d.x, o.x), __fmaf_rn(t, d.y, o.y), __fmaf_rn(t, d.z, o.z), e0, e1);
-    const float near = 4e-6f * (fabsf(t) + fabsf(o.x) + fabsf(o.y) + fabsf(o.z) + e0);
-    bool root = a.refine_root && fabsf(phi - e0) <= near;
+    float t = a.hits[i].t;
+    // The refined t is one end of the last bracket, whose ends are neighbouring
+    // floats with phi >= eps_hit at the lower and phi < eps_hit at the upper one (a
+    // root so near the start that 24 halvings do not get there is marched again).
+    auto below = [&](float s) {
+        float e0, e1;
+        const float phi = field_at<L>(a, __fmaf_rn(s, d.x, o.x), __fmaf_rn(s, d.y, o.y), __fmaf_rn(s, d.z, o.z), e0, e1);
+        return phi < e0;
+    };
+    bool root = false;
+    if (a.refine_root) root = below(t) ? !below(nextafterf(t, -INFINITY)) : below(nextafterf(t, INFINITY));
     if (root) {
         // a hit at the first sample has no bracket, and its t is the march's start
         float ta = ts, tb = te;
