@@ -314,8 +314,8 @@ rt_status rt_trace_sdf(const rt_sdf* sdf, const rt_ray* d_rays, int64_t n, const
                        rt_hit* d_hits, void* stream);
 
 /* The combined query (Eq. 2 and the rules of rt_split_params) for n rays.
- * `params` is read on the host during the call.  With the stage kernels, a
- * closest-hit split call with 0 < m_near < inf runs its near triangle stage
+ * `params` is read on the host during the call.  With the stage kernels (see
+ * rt_tuning.kernel), a closest-hit split call with 0 < m_near < inf runs its near triangle stage
  * and its field stage at the same time, on two streams of the library forked
  * from `stream` and joined back into it by events (calls on one device share
  * these streams; a lock keeps each call's launches together).  The records
@@ -402,7 +402,9 @@ enum { RT_MAX_BATCHES = 16 };
  *   - at most RT_MAX_BATCHES batches, at most 2^31-1 queries in total;
  *   - mode, any_hit, m_near and m_far may differ per batch; max_steps,
  *     hit_eps_vox, min_step_vox and refine_root must be equal in all batches;
- *   - always uses the wavefront stage kernels; the tuning's block, residency,
+ *   - with at most 131,072 queries in all, one launch of one thread per query
+ *     serves the call, unless the tuning's kernel is RT_KERNEL_WAVEFRONT;
+ *     otherwise the wavefront stage kernels do; the tuning's block, residency,
  *     refill and layout apply.
  * Errors: RT_ERR_INVALID_ARG before any work for bad batches. */
 rt_status rt_trace_batches(const rt_scene* scene, const rt_sdf* sdf, const rt_batch* batches, int32_t n_batches,
@@ -429,10 +431,13 @@ rt_status rt_trace_combined_backward(const rt_scene* scene, const rt_sdf* sdf, c
  *                 sub-interval kind, with per-lane refill from a global queue,
  *                 so rays that switch tracer mid-query are regrouped across
  *                 the whole batch; RT_KERNEL_SIMPLE: one thread per query runs
- *                 all its sub-intervals; RT_KERNEL_AUTO (default): the stage
- *                 kernels (on triangles-only calls as well, where they were
- *                 measured at least as fast as one thread per query on GI,
- *                 primary and AO rays).
+ *                 all its sub-intervals; RT_KERNEL_AUTO (default): one
+ *                 thread per query, in one launch, for calls of at most
+ *                 131,072 queries (65,536 if they trace triangles only), the
+ *                 stage kernels for larger ones, on triangles-only calls as
+ *                 well, where they were measured at least as fast on GI,
+ *                 primary and AO rays.  rt_trace_combined_counted and _timed
+ *                 run the stage kernels at every size.
  *   block         threads per block (multiple of 32, 32..1024)
  *   blocks_per_sm persistent grid = SMs x this (0: as many as fit)
  *   refill_min    triangle stages: a warp fetches new queries when at least

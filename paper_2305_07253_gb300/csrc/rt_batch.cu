@@ -331,6 +331,35 @@ __global__ void __maxnreg__(40) k_batch_field(const TraceArgs a, const BatchTabl
     }
 }
 
+// One thread per query: the whole program of its batch, in one launch
+template <int L, bool WIDE>
+__global__ void k_batch_simple(const TraceArgs a, const BatchTable tb)
+{
+    __shared__ BatchEntry stb[RT_MAX_BATCHES];
+    stage_table(tb, stb);
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= a.n) return;
+    const BatchEntry e = stb[find_batch(stb, tb.count, g)];
+    Counts cnt = {0, 0, 0, 0};
+    trace_query<false, L, WIDE>(a, {e.mode, e.any_hit, e.m_near, e.m_far}, e.rays + 2 * (g - e.offset), e.hits + (g - e.offset), cnt);
+}
+
+template <bool WIDE>
+void launch_batch_simple(const TraceArgs& a, const BatchTable& tb, int block, cudaStream_t s)
+{
+    const unsigned nb = (unsigned)((a.n + block - 1) / block);
+    switch (grid_layout_of(a)) {
+    case GL_PLAIN_F32: k_batch_simple<GL_PLAIN_F32, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_PLAIN_F16: k_batch_simple<GL_PLAIN_F16, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_CELLS_F32: k_batch_simple<GL_CELLS_F32, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_CELLS_F16: k_batch_simple<GL_CELLS_F16, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_PAIRS_F32: k_batch_simple<GL_PAIRS_F32, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_PAIRS_F16: k_batch_simple<GL_PAIRS_F16, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    case GL_CASC_F32: k_batch_simple<GL_CASC_F32, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    default: k_batch_simple<GL_CASC_F16, WIDE><<<nb, block, 0, s>>>(a, tb); break;
+    }
+}
+
 struct BatchDevice {
     int sms = 0;
     cudaMemPool_t pool = nullptr;
@@ -432,6 +461,14 @@ extern "C" rt_status rt_trace_batches(const rt_scene* sc, const rt_sdf* sdf, con
     rt_apply_layout(a, tu);
     a.n = total;
     a.counters = nullptr;
+    if (tu.kernel != RT_KERNEL_WAVEFRONT && total <= kSmallCall) {
+        // every query resident at once: the pipeline's launches would cost more
+        // than regrouping gains (rt_launch_trace)
+        if (a.wnodes) launch_batch_simple<true>(a, tb, tu.block, (cudaStream_t)stream);
+        else launch_batch_simple<false>(a, tb, tu.block, (cudaStream_t)stream);
+        RT_CUDA_TRY(cudaGetLastError());
+        return RT_OK;
+    }
     // closest-hit near sub-intervals in some batch: the query order (unless the
     // tuning turns it off) and the concurrent program
     bool near_split = false;

@@ -248,6 +248,11 @@ constexpr int kConcFieldBlocks = RT_CONC_FIELD_BLOCKS;
 constexpr size_t kScratchKept = (size_t)64 << 20;
 rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 
+// Queries up to which RT_KERNEL_AUTO takes one thread per query: about those
+// resident at once (rt_launch_trace has the figures)
+constexpr int64_t kSmallCall = 131072;
+constexpr int64_t kSmallCallTriangles = 65536;  // calls that trace triangles only
+
 // allow_concurrent = false: the stages of a closest-hit split call run in
 // sequence on s (no internal streams), as the pieces of rt_trace_combined_host need
 rt_status rt_launch_trace(const TraceArgs& a, bool counted, cudaStream_t s, StageTiming* timing = nullptr,

@@ -14,7 +14,8 @@
 //     rays that switch tracer mid-query are regrouped across the whole batch
 //     instead of diverging inside a warp.
 //   * simple: one thread per query runs all of its sub-intervals.
-// The default (RT_KERNEL_AUTO) takes the stage kernels.
+// The default (RT_KERNEL_AUTO) takes the stage kernels for large calls and one
+// thread per query for small ones (small_call).
 #include <mutex>
 
 #include "rt_trace_dev.cuh"
@@ -31,61 +32,8 @@ constexpr int kFieldBudget = RT_FIELD_BUDGET;  // march steps between two refill
 constexpr int32_t kRefinePending = RT_TRACER_SDF | 0x100;  // tracer of a record that waits for k_refine
 
 // ---------------------------------------------------------------------------
-// simple kernel: one thread per query
+// simple kernel: one thread per query (trace_query, rt_trace_dev.cuh)
 // ---------------------------------------------------------------------------
-template <bool COUNT, int L, bool WIDE>
-__device__ __forceinline__ void trace_one(const TraceArgs& a, int64_t i, Counts& cnt)
-{
-    const float4 r0 = __ldg(a.rays + 2 * i), r1 = __ldg(a.rays + 2 * i + 1);
-    const float3 o = make_float3(r0.x, r0.y, r0.z), d = make_float3(r1.x, r1.y, r1.z);
-    const float tmin = r0.w, tmax = r1.w;
-    Hit h = {__int_as_float(0x7f800000), -1, 0.f, 0.f};
-    uint32_t flags = 0;
-    int32_t tracer = RT_TRACER_MISS;
-
-    if (!valid_query(o, d, tmin, tmax)) {
-    } else if (a.mode == RT_MODE_BVH) {
-        if (bvh_segment<COUNT, WIDE>(a, o, d, tmin, tmax, a.any_hit, h, flags, cnt)) tracer = RT_TRACER_BVH;
-    } else if (a.mode == RT_MODE_SDF) {
-        March m = sdf_march<COUNT, L>(a, o, d, tmin, tmax, flags, cnt);
-        if (m.hit) {
-            tracer = RT_TRACER_SDF;
-            h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
-        }
-    } else {
-        const Split s = make_split(a, o, d, tmin, tmax);
-        if (a.any_hit) {
-            if (s.field) {
-                March m = sdf_march<COUNT, L>(a, o, d, s.t1, s.t2, flags, cnt);
-                if (m.hit) {
-                    tracer = RT_TRACER_SDF;
-                    h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
-                }
-            }
-            if (tracer == RT_TRACER_MISS && s.near_bvh && bvh_segment<COUNT, WIDE>(a, o, d, tmin, s.t1, true, h, flags, cnt))
-                tracer = RT_TRACER_BVH;
-            if (tracer == RT_TRACER_MISS && s.far_bvh && bvh_segment<COUNT, WIDE>(a, o, d, s.t2, tmax, true, h, flags, cnt))
-                tracer = RT_TRACER_BVH;
-        } else {
-            if (s.near_bvh && bvh_segment<COUNT, WIDE>(a, o, d, tmin, s.t1, false, h, flags, cnt)) tracer = RT_TRACER_BVH;
-            if (tracer == RT_TRACER_MISS && s.field) {
-                March m = sdf_march<COUNT, L>(a, o, d, s.t1, s.t2, flags, cnt);
-                if (m.hit) {
-                    tracer = RT_TRACER_SDF;
-                    h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
-                }
-            }
-            if (tracer == RT_TRACER_MISS && s.far_bvh && bvh_segment<COUNT, WIDE>(a, o, d, s.t2, tmax, false, h, flags, cnt))
-                tracer = RT_TRACER_BVH;
-        }
-    }
-    if (tracer != RT_TRACER_BVH) {
-        h.prim = -1;
-        h.u = h.v = 0.f;
-    }
-    store_hit(a.hits + i, h.t, h.prim, h.u, h.v, tracer, flags);
-}
-
 __device__ __forceinline__ void flush_counts(const TraceArgs& a, const Counts& cnt)
 {
     if (cnt.nodes) atomicAdd(&a.counters[0], (unsigned long long)cnt.nodes);
@@ -99,7 +47,10 @@ __global__ void k_trace(const TraceArgs a)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     Counts cnt = {0, 0, 0, 0};
-    if (i < a.n) trace_one<COUNT, L, WIDE>(a, first_query(a, i), cnt);
+    if (i < a.n) {
+        const int64_t q = first_query(a, i);
+        trace_query<COUNT, L, WIDE>(a, {a.mode, a.any_hit, a.m_near, a.m_far}, a.rays + 2 * q, a.hits + q, cnt);
+    }
     if (COUNT) flush_counts(a, cnt);
 }
 
@@ -766,15 +717,36 @@ rt_status rt_launch_merge_hits(const HitEntry* list, const unsigned* count, int 
     return RT_OK;
 }
 
+// Queries up to which RT_KERNEL_AUTO takes one thread per query.  The stage
+// kernels refill idle lanes and regroup rays between tracers, at the price of up
+// to five launches, a counter reset, scratch and the events between two streams;
+// a call whose queries are all resident at once has nothing to refill.  us a
+// call, stage kernels / one thread per query (frame scene, 256^3; m = 2):
+//   queries        1,000     16,000     128,000    256,000
+//   GI             91 / 57   112 / 80   178 / 145  210 / 201
+//   shadow         114 / 62  122 / 71   208 / 129  210 / 163
+//   field only     65 / 45   91 / 68    152 / 129  177 / 173
+//   GI, cascade    160/150   188/179    233 / 205  268 / 288
+//   triangles only 83 / 80   108/101    151 / 141  251 / 259
+//   primary, triangles only  99 / 96 at 16,000, 113 / 111 at 64,000, 129 / 130 at 128,000
+static int64_t small_call(const TraceArgs& a)
+{
+    const bool triangles_only = a.mode == RT_MODE_BVH || ((a.mode == RT_MODE_SPLIT1 || a.mode == RT_MODE_SPLIT2) && isinf(a.m_near));
+    return triangles_only ? kSmallCallTriangles : kSmallCall;
+}
+
 rt_status rt_launch_trace(const TraceArgs& a0, bool counted, cudaStream_t s, StageTiming* timing,
                           bool allow_concurrent)
 {
     const rt_tuning& tu = rt_current_tuning();
     TraceArgs a = a0;
     rt_apply_layout(a, tu);
-    // AUTO: the stage kernels for every call; on triangles-only calls too they
-    // were measured at least as fast as one thread per query on every ray kind
-    const bool wavefront = tu.kernel == RT_KERNEL_WAVEFRONT || tu.kernel == RT_KERNEL_AUTO;
+    // AUTO: one thread per query, in one launch, where all queries of the call are
+    // resident at once; otherwise the stage kernels.  Calls that count or time
+    // the stages always run them.
+    const bool wavefront = tu.kernel == RT_KERNEL_WAVEFRONT ||
+                           (tu.kernel == RT_KERNEL_AUTO && (counted || timing || a.n > small_call(a)));
+    if (!wavefront && tu.kernel == RT_KERNEL_AUTO) a.ob.bits = 0;  // the order costs a launch, more than it gains here
     if (wavefront)
         return counted ? run_wavefront<true>(a, tu, s, timing, allow_concurrent)
                        : run_wavefront<false>(a, tu, s, timing, allow_concurrent);

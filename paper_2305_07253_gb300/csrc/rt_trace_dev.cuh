@@ -815,6 +815,70 @@ __device__ __forceinline__ void store_hit(rt_hit* out, float t, int32_t prim, fl
     p[2] = make_float2(__int_as_float(tracer), __uint_as_float(flags));
 }
 
+// How a query is split and processed (rt_split_params)
+struct QueryProgram {
+    int32_t mode, any_hit;
+    float m_near, m_far;
+};
+
+// A whole query in one thread: all sub-intervals of its program, in the order of
+// Section 2, and its record
+template <bool COUNT, int L, bool WIDE>
+__device__ __forceinline__ void trace_query(const TraceArgs& a, const QueryProgram& pr, const float4* ray, rt_hit* out,
+                                            Counts& cnt)
+{
+    const float4 r0 = __ldg(ray), r1 = __ldg(ray + 1);
+    const float3 o = make_float3(r0.x, r0.y, r0.z), d = make_float3(r1.x, r1.y, r1.z);
+    const float tmin = r0.w, tmax = r1.w;
+    Hit h = {__int_as_float(0x7f800000), -1, 0.f, 0.f};
+    uint32_t flags = 0;
+    int32_t tracer = RT_TRACER_MISS;
+
+    if (!valid_query(o, d, tmin, tmax)) {
+    } else if (pr.mode == RT_MODE_BVH) {
+        if (bvh_segment<COUNT, WIDE>(a, o, d, tmin, tmax, pr.any_hit, h, flags, cnt)) tracer = RT_TRACER_BVH;
+    } else if (pr.mode == RT_MODE_SDF) {
+        March m = sdf_march<COUNT, L>(a, o, d, tmin, tmax, flags, cnt);
+        if (m.hit) {
+            tracer = RT_TRACER_SDF;
+            h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
+        }
+    } else {
+        float hn, hf;
+        split_voxels(a, o, d, tmin, tmax, hn, hf);
+        const Split s = make_split(pr.mode, pr.m_near, pr.m_far, hn, hf, tmin, tmax);
+        if (pr.any_hit) {
+            if (s.field) {
+                March m = sdf_march<COUNT, L>(a, o, d, s.t1, s.t2, flags, cnt);
+                if (m.hit) {
+                    tracer = RT_TRACER_SDF;
+                    h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
+                }
+            }
+            if (tracer == RT_TRACER_MISS && s.near_bvh && bvh_segment<COUNT, WIDE>(a, o, d, tmin, s.t1, true, h, flags, cnt))
+                tracer = RT_TRACER_BVH;
+            if (tracer == RT_TRACER_MISS && s.far_bvh && bvh_segment<COUNT, WIDE>(a, o, d, s.t2, tmax, true, h, flags, cnt))
+                tracer = RT_TRACER_BVH;
+        } else {
+            if (s.near_bvh && bvh_segment<COUNT, WIDE>(a, o, d, tmin, s.t1, false, h, flags, cnt)) tracer = RT_TRACER_BVH;
+            if (tracer == RT_TRACER_MISS && s.field) {
+                March m = sdf_march<COUNT, L>(a, o, d, s.t1, s.t2, flags, cnt);
+                if (m.hit) {
+                    tracer = RT_TRACER_SDF;
+                    h.t = (a.refine_root && !isnan(m.t_prev)) ? refine<L>(a, o, d, m.t_prev, m.t) : m.t;
+                }
+            }
+            if (tracer == RT_TRACER_MISS && s.far_bvh && bvh_segment<COUNT, WIDE>(a, o, d, s.t2, tmax, false, h, flags, cnt))
+                tracer = RT_TRACER_BVH;
+        }
+    }
+    if (tracer != RT_TRACER_BVH) {
+        h.prim = -1;
+        h.u = h.v = 0.f;
+    }
+    store_hit(out, h.t, h.prim, h.u, h.v, tracer, flags);
+}
+
 // Append the lanes with `hit` set to a near-hit list (one atomic per warp):
 // the record dst, and the hit found (prim kFlagsOnly: none, flags only).
 __device__ __forceinline__ void append_hit_entry(HitEntry* list, unsigned* count, bool hit, rt_hit* dst,
