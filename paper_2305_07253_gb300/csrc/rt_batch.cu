@@ -232,6 +232,7 @@ __global__ void __maxnreg__(40) k_batch_field(const TraceArgs a, const BatchTabl
 {
     __shared__ BatchEntry stb[RT_MAX_BATCHES];
     stage_table(tb, stb);
+    stage_levels<L>(a);
     const unsigned n_in = pp.in_items ? *pp.in_count : pp.n_first;
     rt_hit* hits = nullptr;
     bool has_next = false;
@@ -337,6 +338,7 @@ __global__ void k_batch_simple(const TraceArgs a, const BatchTable tb)
 {
     __shared__ BatchEntry stb[RT_MAX_BATCHES];
     stage_table(tb, stb);
+    stage_levels<L>(a);
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= a.n) return;
     const BatchEntry e = stb[find_batch(stb, tb.count, g)];

@@ -47,6 +47,7 @@ __global__ void k_trace(const TraceArgs a)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     Counts cnt = {0, 0, 0, 0};
+    stage_levels<L>(a);
     if (i < a.n) {
         const int64_t q = first_query(a, i);
         trace_query<COUNT, L, WIDE>(a, {a.mode, a.any_hit, a.m_near, a.m_far}, a.rays + 2 * q, a.hits + q, cnt);
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(256) k_merge_hits(const HitEntry* __restrict__
 template <bool COUNT, int L>
 __global__ void __maxnreg__(RT_FIELD_REGS) k_stage_field(const TraceArgs a, const StageArgs st)
 {
+    stage_levels<L>(a);
     const unsigned n_in = st.first ? (unsigned)a.n : *st.in_count;
     Counts cnt = {0, 0, 0, 0};
     bool drained = false, live = false, more = false;
@@ -307,6 +309,7 @@ __global__ void __maxnreg__(RT_FIELD_REGS) k_stage_field(const TraceArgs a, cons
 template <int L>
 __global__ void __launch_bounds__(128) k_refine(const TraceArgs a)
 {
+    stage_levels<L>(a);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     rt_hit* h = a.hits + i;

@@ -610,27 +610,54 @@ __device__ __forceinline__ float trilinear(const TraceArgs& a, float px, float p
 // closed box holds p (the coarsest outside all boxes; a NaN point is outside
 // every box); trilinear sample of that level from its cells
 // ---------------------------------------------------------------------------
+// The levels nest, so the level is the number of finer ones whose box does not
+// hold p: no branches, no lane waits for another's search.
 __device__ __forceinline__ int casc_level(const TraceArgs& a, float px, float py, float pz)
 {
     int k = 0;
-    for (; k < a.levels - 1; ++k) {
-        const CascLevel& v = a.lv[k];
-        if (px >= v.lo[0] && px <= v.hi[0] && py >= v.lo[1] && py <= v.hi[1] && pz >= v.lo[2] && pz <= v.hi[2])
-            break;
+#pragma unroll
+    for (int j = 0; j < RT_MAX_LEVELS - 1; ++j) {
+        if (j >= a.levels - 1) break;  // the same for all lanes
+        const CascLevel& v = a.lv[j];
+        const bool in = px >= v.lo[0] && px <= v.hi[0] && py >= v.lo[1] && py <= v.hi[1] && pz >= v.lo[2] && pz <= v.hi[2];
+        k += in ? 0 : 1;
     }
     return k;
+}
+
+// What a march step needs of a level, staged in shared memory at the start of a
+// kernel that marches through a cascade: lanes at different levels read their rows
+// together, where reads of the kernel's parameters by lane would take turns.
+// Row k: lo x, y, z, 1/h | eps_hit, eps_min, -, -.
+__device__ __forceinline__ float4* level_table()
+{
+    __shared__ float4 rows[2 * RT_MAX_LEVELS];
+    return rows;
+}
+template <int L>
+__device__ __forceinline__ void stage_levels(const TraceArgs& a)
+{
+    if constexpr (is_cascade(L)) {
+        float4* t = level_table();
+        if (threadIdx.x < RT_MAX_LEVELS && (int)threadIdx.x < a.levels) {
+            const CascLevel& v = a.lv[threadIdx.x];
+            t[2 * threadIdx.x] = make_float4(v.lo[0], v.lo[1], v.lo[2], v.ih);
+            t[2 * threadIdx.x + 1] = make_float4(v.eps_hit, v.eps_min, 0.f, 0.f);
+        }
+        __syncthreads();
+    }
 }
 
 // the cell of level k that holds p (its index in the cell copy) and p's fractions in it
 __device__ __forceinline__ int64_t casc_locate(const TraceArgs& a, int k, float px, float py, float pz, float f[3])
 {
-    const CascLevel& lv = a.lv[k];
-    const float p[3] = {px, py, pz};
+    const float4 row = level_table()[2 * k];
+    const float p[3] = {px, py, pz}, lo[3] = {row.x, row.y, row.z};
     const float top = (float)(a.gn[0] - 1);
     int i0[3];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
-        float u = __fmul_rn(__fsub_rn(p[ax], lv.lo[ax]), lv.ih);
+        float u = __fmul_rn(__fsub_rn(p[ax], lo[ax]), row.w);
         u = fminf(fmaxf(u, 0.f), top);
         int ii = (int)floorf(u);
         if (ii > a.gn[0] - 2) ii = a.gn[0] - 2;
@@ -658,8 +685,9 @@ __device__ __forceinline__ float field_at(const TraceArgs& a, float px, float py
 {
     if constexpr (is_cascade(L)) {
         const int k = casc_level(a, px, py, pz);
-        eps_hit = a.lv[k].eps_hit;
-        eps_min = a.lv[k].eps_min;
+        const float2 e = *reinterpret_cast<const float2*>(level_table() + 2 * k + 1);
+        eps_hit = e.x;
+        eps_min = e.y;
         return casc_trilinear<L>(a, k, px, py, pz);
     } else {
         eps_hit = a.eps_hit;
