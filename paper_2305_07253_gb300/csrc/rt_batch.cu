@@ -554,7 +554,7 @@ extern "C" rt_status rt_trace_batches(const rt_scene* sc, const rt_sdf* sdf, con
         pp.hit_list = list;
         pp.hit_count = hit_count;
         rt_tuning tk = tu;
-        if (conc && tu.blocks_per_sm == 0 && !helper && kk <= 1) tk.blocks_per_sm = kk == 0 ? kConcNearBlocks : kConcFieldBlocks;
+        if (conc && tu.blocks_per_sm == 0 && !helper && kk <= 1) tk.blocks_per_sm = kk == 0 ? kConcNearBatch : kConcFieldBatch;
         const cudaStream_t sk = !conc ? s : (k == 0 ? s_tri : s_field);
         const TraceArgs& ak = kk == 1 ? af : a;
         if (kk == 1 && need_grid) {

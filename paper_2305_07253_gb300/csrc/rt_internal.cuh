@@ -228,19 +228,16 @@ rt_status rt_conc_streams(ConcStreams*& out);
 rt_status rt_launch_merge_hits(const HitEntry* list, const unsigned* count, int sms, cudaStream_t s);
 // Resident blocks of 128 threads per SM of the two concurrent stages when the
 // tuning leaves them free.  Both kernels are persistent, so their blocks must
-// fit in an SM side by side (registers: near 2 x 128 x 56 (64 for the batch
-// kernel) + field 9 x 128 x 40, at most 62,464 of 65,536), or the later launch
-// waits for the earlier one's end.  Measured on the 1080p GI workload, whole
-// call: near 2 + field 9 0.595 ms, 3 + 9 0.608, 2 + 10 0.603, 2 + 8 0.611,
-// 4 + 7 0.661, 1 + 11 1.015; the stages in sequence 0.662.
-#ifndef RT_CONC_NEAR_BLOCKS
-#define RT_CONC_NEAR_BLOCKS 2
-#endif
-#ifndef RT_CONC_FIELD_BLOCKS
-#define RT_CONC_FIELD_BLOCKS 9
-#endif
-constexpr int kConcNearBlocks = RT_CONC_NEAR_BLOCKS;
-constexpr int kConcFieldBlocks = RT_CONC_FIELD_BLOCKS;
+// fit in an SM side by side (registers: near 56, 64 for the batch kernel, field
+// 40, times 128 threads, at most 65,536), or the later launch waits for the
+// earlier one's end.  Measured, ms a call, near + field blocks: 1080p GI on one
+// grid (256^3) 2 + 10 0.578, 2 + 9 0.594, 3 + 8 0.602, 4 + 7 0.649; on a 5 x 64^3
+// cascade, whose near sub-intervals are several times longer, 5 + 5 0.806, 4 + 7
+// 0.813, 3 + 8 0.837, 2 + 9 0.859; a mixed frame 3 + 8 1.946, 4 + 7 1.971, 2 + 9
+// 1.992, 5 + 6 2.211.
+constexpr int kConcNearBlocks = 2, kConcFieldBlocks = 10;
+constexpr int kConcNearCascade = 4, kConcFieldCascade = 7;
+constexpr int kConcNearBatch = 3, kConcFieldBatch = 8;
 
 // Device scratch in stream order (free it with cudaFreeAsync).  Up to
 // kScratchKept bytes come from the library's pool, which keeps what is freed;

@@ -514,8 +514,8 @@ rt_status run_concurrent(const TraceArgs& a, const int kinds[3], int n_st, const
     if (e != cudaSuccess) rs = rt_cuda_fail(e, "concurrent program set-up");
     rt_tuning tn = tu, tf = tu;
     if (tu.blocks_per_sm == 0) {
-        tn.blocks_per_sm = kConcNearBlocks;
-        tf.blocks_per_sm = kConcFieldBlocks;
+        tn.blocks_per_sm = a.levels > 0 ? kConcNearCascade : kConcNearBlocks;
+        tf.blocks_per_sm = a.levels > 0 ? kConcFieldCascade : kConcFieldBlocks;
     }
     // near stream: the order, then the near stage
     TraceArgs ao = a;
