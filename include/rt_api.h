@@ -277,12 +277,11 @@ rt_status rt_cascade_recenter(const rt_scene* scene, rt_sdf* sdf, const float ce
 
 /* The combined query of rt_trace_combined for rays and hit records in host
  * memory: the rays are copied to d_rays, traced, and the records copied back
- * to h_hits, in `chunks` pieces (0: 4; 1..64; from 3 pieces on, the first and
- * last are half as large as the others) pipelined over two copy streams and
- * up to four compute streams owned by the library, so that the upload of one
- * piece, the traces of the previous ones and the download of the one before
- * overlap.  The
- * paper's queries start on the GPU (Section 3); this call serves callers whose
+ * to h_hits, in `chunks` pieces (0: 2 to 6 by n; 1..64; from 3 pieces on, the
+ * first and last are half as large as the others) pipelined over two copy streams
+ * and up to four compute streams owned by the library (each with its own pair for
+ * concurrent programs), so that the upload of one piece, the traces of the
+ * previous ones and the download of the one before overlap.  The paper's queries start on the GPU (Section 3); this call serves callers whose
  * rays live in host memory.
  *   h_rays, h_hits  host memory of n rays / records; page-locked memory
  *                   (cudaHostAlloc, torch pin_memory) is needed for the copies

@@ -475,13 +475,9 @@ extern "C" rt_status rt_sdf_sites(const rt_scene* sc, const rt_sdf* sdf, int32_t
     return rt_launch_df_sites(sc, sdf, stage, d_sites, (cudaStream_t)stream);
 }
 
-// allow_order = false: trace in input order whatever the tuning, and the
-// stages in sequence on `stream` (the pieces of rt_trace_combined_host, whose
-// pipeline an extra kernel per piece slows down, and whose pieces run on
-// streams of their own)
 static rt_status trace_common(const rt_scene* sc, const rt_sdf* sdf, const rt_ray* rays, int64_t n,
                               const rt_split_params* p, rt_hit* hits, unsigned long long* counters,
-                              void* stream, StageTiming* timing = nullptr, bool allow_order = true)
+                              void* stream, StageTiming* timing = nullptr, int conc_set = 0)
 {
     rt_status st = check_params(p);
     if (st != RT_OK) return st;
@@ -506,8 +502,10 @@ static rt_status trace_common(const rt_scene* sc, const rt_sdf* sdf, const rt_ra
     a.hits = hits;
     a.n = n;
     a.counters = counters;
-    if (!allow_order || !rt_order_applies(*p)) a.ob.bits = 0;
-    return rt_launch_trace(a, counters != nullptr, (cudaStream_t)stream, timing, allow_order);
+    // (no query order in a piece of rt_trace_combined_host: its kernel would wait for
+    // SMs that the other pieces' persistent kernels hold)
+    if (conc_set > 0 || !rt_order_applies(*p)) a.ob.bits = 0;
+    return rt_launch_trace(a, counters != nullptr, (cudaStream_t)stream, timing, conc_set);
 }
 
 extern "C" rt_status rt_trace_combined_timed(const rt_scene* sc, const rt_sdf* sdf, const rt_ray* rays, int64_t n,
@@ -570,6 +568,7 @@ extern "C" rt_status rt_trace_combined(const rt_scene* sc, const rt_sdf* sdf, co
 namespace {
 constexpr int kMaxChunks = 64;
 constexpr int kComputeStreams = 4;
+static_assert(kComputeStreams < kConcSets, "a set of streams for the pieces of each compute stream");
 struct HostPipe {
     cudaStream_t in = nullptr, out = nullptr;
     cudaStream_t comp[kComputeStreams] = {};
@@ -614,7 +613,14 @@ extern "C" rt_status rt_trace_combined_host(const rt_scene* sc, const rt_sdf* sd
     if (n > 0 && (!h_rays || !h_hits)) return rt_fail(RT_ERR_INVALID_ARG, "null host ray or hit buffer");
     if (chunks < 0 || chunks > kMaxChunks) return rt_fail(RT_ERR_INVALID_ARG, "chunks %d not in 0..%d", chunks, kMaxChunks);
     if (n == 0) return RT_OK;
-    if (chunks == 0) chunks = 4;
+    // More pieces hide more of the copies and pay more of the host's calls (about
+    // 30 us a piece) and of the pieces' tails.  Frame scene, 256^3, us end to end,
+    // GI / shadow / triangles only, by pieces:
+    //   2,073,600 queries  4  931 / 856 / 1404   6  878 / 803 / 1393   8  882 (GI)
+    //   400,000            4  352 / 331 / 410    5  307 / 256 / 403    6  335 / 269 / 401
+    //   200,000            4  211 / 190 / 275    5  267 / 213 / 330
+    //   32,000             2  101 / 110 / 135    4  101 / 109 / 134    6  168 / 154 / 223
+    if (chunks == 0) chunks = n <= 65536 ? 2 : (n <= 262144 ? 4 : (n < 1048576 ? 5 : 6));
     if (chunks > n) chunks = (int32_t)n;
     // the library's copy streams are shared by all callers on this device
     std::lock_guard<std::mutex> lk(g_pipe_mu);
@@ -643,7 +649,7 @@ extern "C" rt_status rt_trace_combined_host(const rt_scene* sc, const rt_sdf* sd
         RT_CUDA_TRY(cudaMemcpyAsync(d_rays + b, h_rays + b, (size_t)m * sizeof(rt_ray), cudaMemcpyHostToDevice, p->in));
         RT_CUDA_TRY(cudaEventRecord(p->ev_in[c], p->in));
         RT_CUDA_TRY(cudaStreamWaitEvent(cs, p->ev_in[c], 0));
-        st = trace_common(sc, sdf, d_rays + b, m, params, d_hits + b, nullptr, cs, nullptr, false);
+        st = trace_common(sc, sdf, d_rays + b, m, params, d_hits + b, nullptr, cs, nullptr, 1 + c % ncomp);
         if (st != RT_OK) return st;
         RT_CUDA_TRY(cudaEventRecord(p->ev_tr[c], cs));
         RT_CUDA_TRY(cudaStreamWaitEvent(p->out, p->ev_tr[c], 0));

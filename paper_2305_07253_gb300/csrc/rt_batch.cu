@@ -504,7 +504,7 @@ extern "C" rt_status rt_trace_batches(const rt_scene* sc, const rt_sdf* sdf, con
     cudaStream_t s_tri = s, s_field = s;  // the streams of the first two launches
     if (conc && rs == RT_OK) {
         lk.lock();
-        rs = rt_conc_streams(cs);
+        rs = rt_conc_streams(0, cs);
         if (rs == RT_OK) {
             e = cudaEventRecord(cs->fork, s);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(cs->near, cs->fork, 0);

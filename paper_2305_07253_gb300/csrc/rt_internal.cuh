@@ -223,7 +223,10 @@ struct ConcStreams {
     bool ready = false;
 };
 std::mutex& rt_conc_mutex();
-rt_status rt_conc_streams(ConcStreams*& out);
+// set 0: calls and batches; sets 1 .. kConcSets - 1: the pieces of
+// rt_trace_combined_host, which would wait for one another on shared streams
+constexpr int kConcSets = 5;
+rt_status rt_conc_streams(int set, ConcStreams*& out);
 // k_merge_hits over the *count entries of list, on s
 rt_status rt_launch_merge_hits(const HitEntry* list, const unsigned* count, int sms, cudaStream_t s);
 // Resident blocks of 128 threads per SM of the two concurrent stages when the
@@ -250,10 +253,9 @@ rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 constexpr int64_t kSmallCall = 131072;
 constexpr int64_t kSmallCallTriangles = 65536;  // calls that trace triangles only
 
-// allow_concurrent = false: the stages of a closest-hit split call run in
-// sequence on s (no internal streams), as the pieces of rt_trace_combined_host need
+// conc_set: the set of library streams a concurrent program of this call uses
 rt_status rt_launch_trace(const TraceArgs& a, bool counted, cudaStream_t s, StageTiming* timing = nullptr,
-                          bool allow_concurrent = true);
+                          int conc_set = 0);
 rt_status rt_launch_backward(const TraceArgs& a, const float* grad_t, float* grad_grid, cudaStream_t s);
 rt_status rt_build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt, cudaStream_t s,
                          rt_scene* out);

@@ -442,7 +442,7 @@ int32_t public_kind(int k)
 // Streams and events of the concurrent programs, one set per device, and the
 // lock that keeps one call's fork-to-join sequence of launches together.
 std::mutex g_conc_mu;
-ConcStreams g_conc[64];
+ConcStreams g_conc[64][kConcSets];
 
 // Work counters sit 128 bytes apart: atomics of different counters, from one
 // kernel or from two running side by side, then never share an L2 line.
@@ -490,11 +490,11 @@ StageArgs stage_args(int kind, const rt_tuning& tu)
 // those of the stages run in sequence.
 template <bool COUNT>
 rt_status run_concurrent(const TraceArgs& a, const int kinds[3], int n_st, const rt_tuning& tu, DeviceInfo* dev,
-                         cudaStream_t s, Marks& marks)
+                         cudaStream_t s, Marks& marks, int conc_set)
 {
     ConcStreams* cs = nullptr;
     std::lock_guard<std::mutex> lk(g_conc_mu);
-    rt_status st = rt_conc_streams(cs);
+    rt_status st = rt_conc_streams(conc_set, cs);
     if (st != RT_OK) return st;
     const bool far = n_st > 2;
     const size_t counters_bytes = 8 * kCtrStride * sizeof(unsigned);
@@ -600,8 +600,7 @@ rt_status run_concurrent(const TraceArgs& a, const int kinds[3], int n_st, const
 }
 
 template <bool COUNT>
-rt_status run_wavefront(const TraceArgs& a, const rt_tuning& tu, cudaStream_t s, StageTiming* timing,
-                        bool allow_concurrent)
+rt_status run_wavefront(const TraceArgs& a, const rt_tuning& tu, cudaStream_t s, StageTiming* timing, int conc_set)
 {
     DeviceInfo* dev = nullptr;
     rt_status st = device_info(dev);
@@ -613,8 +612,8 @@ rt_status run_wavefront(const TraceArgs& a, const rt_tuning& tu, cudaStream_t s,
     if (timing) timing->n_launches = 0;
     // closest-hit split calls: the near and field stages at the same time (not
     // with m_near = +inf, where the field sub-interval is empty for every query)
-    if (allow_concurrent && n_st >= 2 && kinds[0] == ST_BVH_NEAR && !a.any_hit && !isinf(a.m_near))
-        return run_concurrent<COUNT>(a, kinds, n_st, tu, dev, s, marks);
+    if (n_st >= 2 && kinds[0] == ST_BVH_NEAR && !a.any_hit && !isinf(a.m_near))
+        return run_concurrent<COUNT>(a, kinds, n_st, tu, dev, s, marks, conc_set);
     // scratch: counters (fetch x3, queue sizes x2), the query order, and two
     // ping-pong queues
     const size_t counters_bytes = 8 * kCtrStride * sizeof(unsigned);
@@ -689,12 +688,12 @@ rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s)
     return RT_OK;
 }
 
-rt_status rt_conc_streams(ConcStreams*& out)
+rt_status rt_conc_streams(int set, ConcStreams*& out)
 {
     int dev = 0;
     RT_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return rt_fail(RT_ERR_INVALID_ARG, "device %d out of range", dev);
-    ConcStreams& c = g_conc[dev];
+    ConcStreams& c = g_conc[dev][set];
     if (!c.ready) {
         // the near stream at the highest priority: when both stages have blocks
         // waiting for room (after the order kernel), the near stage's are placed
@@ -739,7 +738,7 @@ static int64_t small_call(const TraceArgs& a)
 }
 
 rt_status rt_launch_trace(const TraceArgs& a0, bool counted, cudaStream_t s, StageTiming* timing,
-                          bool allow_concurrent)
+                          int conc_set)
 {
     const rt_tuning& tu = rt_current_tuning();
     TraceArgs a = a0;
@@ -751,8 +750,8 @@ rt_status rt_launch_trace(const TraceArgs& a0, bool counted, cudaStream_t s, Sta
                            (tu.kernel == RT_KERNEL_AUTO && (counted || timing || a.n > small_call(a)));
     if (!wavefront && tu.kernel == RT_KERNEL_AUTO) a.ob.bits = 0;  // the order costs a launch, more than it gains here
     if (wavefront)
-        return counted ? run_wavefront<true>(a, tu, s, timing, allow_concurrent)
-                       : run_wavefront<false>(a, tu, s, timing, allow_concurrent);
+        return counted ? run_wavefront<true>(a, tu, s, timing, conc_set)
+                       : run_wavefront<false>(a, tu, s, timing, conc_set);
     const int64_t blocks = (a.n + tu.block - 1) / tu.block;
     if (blocks > 0x7fffffffLL) return rt_fail(RT_ERR_INVALID_ARG, "too many rays");
     Marks marks{timing};
