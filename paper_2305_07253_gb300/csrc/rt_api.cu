@@ -236,12 +236,7 @@ extern "C" rt_status rt_scene_export(const rt_scene* sc, void* d_nodes, void* d_
 extern "C" rt_status rt_scene_destroy(rt_scene* sc)
 {
     if (!sc) return RT_OK;
-    cudaFree(sc->nodes);
-    cudaFree(sc->tris);
-    cudaFree(sc->pn);
-    cudaFree(sc->slot);
-    cudaFree(sc->wnodes);
-    cudaFree(sc->wtris);
+    if (sc->block) cudaFree(sc->block);
     delete sc;
     return RT_OK;
 }

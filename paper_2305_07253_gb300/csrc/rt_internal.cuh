@@ -68,6 +68,7 @@ struct rt_scene {
     int32_t wide_depth;
     float lo[3], hi[3];
     int64_t bytes;
+    void* block;    // the one allocation that holds all of the above
 };
 
 struct rt_sdf {
@@ -260,12 +261,58 @@ rt_status rt_launch_backward(const TraceArgs& a, const float* grad_t, float* gra
 rt_status rt_build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt, cudaStream_t s,
                          rt_scene* out);
 rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, cudaStream_t s);
+// Arrays that share one allocation: counted first (base null), then handed out.
+struct BuildArena {
+    char* base = nullptr;
+    size_t at = 0, size = 0;
+    template <class T>
+    T* take(int64_t count)
+    {
+        T* p = base ? reinterpret_cast<T*>(base + at) : nullptr;
+        at += ((size_t)(count > 0 ? count : 1) * sizeof(T) + 255) & ~(size_t)255;
+        if (at > size) size = at;
+        return p;
+    }
+};
+
+// Surface-area costs of the tree (rt_treelet.cu), every rounding written out: the
+// restructured tree must not depend on how a compiler contracts these sums in one
+// place or another (an ulp decides between two topologies of nearly equal cost).
+namespace rttree {
+constexpr float kCostNode = 1.2f;  // visiting a node ...
+constexpr float kCostTri = 1.0f;   // ... and testing a triangle
+__device__ __forceinline__ float half_area(float4 lo, float4 hi)
+{
+    const float dx = __fsub_rn(hi.x, lo.x), dy = __fsub_rn(hi.y, lo.y), dz = __fsub_rn(hi.z, lo.z);
+    return __fmaf_rn(dz, dx, __fmaf_rn(dx, dy, __fmul_rn(dy, dz)));
+}
+__device__ __forceinline__ float node_cost(float4 lo, float4 hi, float c0, float c1)
+{
+    return __fadd_rn(__fmaf_rn(kCostNode, half_area(lo, hi), c0), c1);
+}
+}  // namespace rttree
+
+// workspaces of the restructuring and of the wide tree's collapse
+struct TreeletScratch {
+    int* visit;      // one per internal node
+    int* count;
+    int32_t* pos;    // one per leaf, as the rest
+    int32_t* order2;
+    int32_t* par_l2;
+    float4 *llo2, *lhi2;
+};
+struct WideScratch {
+    int2* items[2];     // (binary node, wide node) pairs of one level
+    unsigned* counters;
+};
+constexpr int kWideCounters = 4 + 260;  // nodes, triangles, error, -; then the items of each level
 rt_status rt_build_wide(rt_scene* sc, const int2* child, const int2* range, const float4* node_lo,
                         const float4* node_hi, const float4* leaf_lo, const float4* leaf_hi, float pad,
-                        cudaStream_t s);
+                        const WideScratch& ws, cudaStream_t s);
 rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s);
 rt_status rt_treelet_optimise(int64_t nt, int passes, int2* child, int2* range, int32_t* par_i, int32_t* par_l,
-                              int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, cudaStream_t s);
+                              int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, float* cost,
+                              const TreeletScratch& ws, cudaStream_t s);
 rt_status rt_fill_trace_args(TraceArgs& a, const rt_scene* sc, const rt_sdf* sdf, const rt_split_params* p);
 void rt_cascade_geometry(const rt_sdf* sdf, int k, float lo[3], float hi[3], float* h, float* ih);
 rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, const void* keep, const int32_t shift[3],

@@ -182,9 +182,10 @@ __device__ __forceinline__ void tri_box(const float* V, const int32_t* F, int32_
 }
 
 // leaf boxes (sorted order), then walk up; the second arrival at a node merges
+// boxes and costs
 __global__ void k_refit(const float* V, const int32_t* F, const int32_t* order, int64_t n, const int2* child,
                         const int32_t* parent_int, const int32_t* parent_leaf, float4* leaf_lo, float4* leaf_hi,
-                        float4* node_lo, float4* node_hi, int* visit)
+                        float4* node_lo, float4* node_hi, float* cost, int* visit)
 {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -202,8 +203,13 @@ __global__ void k_refit(const float* V, const int32_t* F, const int32_t* order, 
         float4 h0 = c.x < 0 ? __ldcg(&leaf_hi[~c.x]) : __ldcg(&node_hi[c.x]);
         float4 l1 = c.y < 0 ? __ldcg(&leaf_lo[~c.y]) : __ldcg(&node_lo[c.y]);
         float4 h1 = c.y < 0 ? __ldcg(&leaf_hi[~c.y]) : __ldcg(&node_hi[c.y]);
-        node_lo[node] = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
-        node_hi[node] = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
+        const float4 nl = make_float4(fminf(l0.x, l1.x), fminf(l0.y, l1.y), fminf(l0.z, l1.z), 0.f);
+        const float4 nh = make_float4(fmaxf(h0.x, h1.x), fmaxf(h0.y, h1.y), fmaxf(h0.z, h1.z), 0.f);
+        node_lo[node] = nl;
+        node_hi[node] = nh;
+        // the subtree's surface-area cost, which the restructuring starts from
+        cost[node] = rttree::node_cost(nl, nh, c.x < 0 ? rttree::kCostTri * rttree::half_area(l0, h0) : __ldcg(&cost[c.x]),
+                                       c.y < 0 ? rttree::kCostTri * rttree::half_area(l1, h1) : __ldcg(&cost[c.y]));
         __threadfence();
         node = parent_int[node];
     }
@@ -322,53 +328,90 @@ __global__ void k_pack_pn(const int32_t* F, const int32_t* order, int64_t n, con
     }
 }
 
-// scoped device allocation released when the build returns
-struct DevBuf {
-    void* p = nullptr;
-    ~DevBuf() { if (p) cudaFree(p); }
-    template <class T>
-    T* as() { return static_cast<T*>(p); }
-};
-
 inline unsigned grid_for(int64_t n) { return (unsigned)((n + kBlock - 1) / kBlock); }
 
 }  // namespace
 
-#define ALLOC(buf, bytes) RT_CUDA_TRY(cudaMalloc(&(buf).p, (size_t)(bytes) > 0 ? (size_t)(bytes) : 16))
+namespace {
 
-rt_status rt_build_scene(const float* V, int64_t nv, const int32_t* F, int64_t nt, cudaStream_t s, rt_scene* sc)
+// Everything the build needs for a while, in one allocation: 25 allocations of
+// their own and their releases (40 to 300 us each, a release waits for the device)
+// and a synchronisation per level of the wide tree were 3 of 13.3 ms (2,050,412
+// triangles).
+struct Work {
+    int32_t* order;  // triangles in leaf order: outlives the first phase
+    // first phase: the trees
+    float4* cen;
+    int *bounds, *depth, *range;
+    uint64_t *keys, *keys2;
+    int32_t *vals, *par_i, *par_l;
+    int2 *child, *nrange;
+    float4 *llo, *lhi, *nlo, *nhi;
+    float* cost;
+    char* sort1;
+    TreeletScratch tl;
+    WideScratch wide;
+    // second phase: the pseudonormals, in the first phase's space
+    float4 *fn, *en;
+    float* vpn;
+    uint64_t *ek, *ek2;
+    int32_t *ev, *ev2;
+    char* sort2;
+};
+
+void lay_out(BuildArena& A, Work& w, int64_t nt, int64_t nv, size_t sort1, size_t sort2)
 {
-    sc->n_tris = nt;
-    sc->n_verts = nv;
-    sc->n_nodes = nt - 1;
-    DevBuf cen, bounds, keys, keys2, vals, vals2, child, par_i, par_l, llo, lhi, nlo, nhi, visit, depth, tmp;
-    DevBuf fn, vpn, ek, ek2, ev, ev2, en;
-    ALLOC(cen, nt * sizeof(float4));
-    ALLOC(bounds, 12 * sizeof(int));
-    ALLOC(keys, nt * sizeof(uint64_t));
-    ALLOC(keys2, nt * sizeof(uint64_t));
-    ALLOC(vals, nt * sizeof(int32_t));
-    ALLOC(vals2, nt * sizeof(int32_t));
-    ALLOC(child, (nt - 1) * sizeof(int2));
-    DevBuf nrange;
-    ALLOC(nrange, (nt - 1) * sizeof(int2));
-    ALLOC(par_i, (nt - 1) * sizeof(int32_t));
-    ALLOC(par_l, nt * sizeof(int32_t));
-    ALLOC(llo, nt * sizeof(float4));
-    ALLOC(lhi, nt * sizeof(float4));
-    ALLOC(nlo, (nt - 1) * sizeof(float4));
-    ALLOC(nhi, (nt - 1) * sizeof(float4));
-    ALLOC(visit, (nt - 1) * sizeof(int));
-    ALLOC(depth, sizeof(int));
+    const int64_t ni = nt > 1 ? nt - 1 : 1;
+    A.at = 0;
+    w.order = A.take<int32_t>(nt);
+    const size_t phase = A.at;
+    w.cen = A.take<float4>(nt);
+    w.bounds = A.take<int>(12);
+    w.depth = A.take<int>(1);
+    w.range = A.take<int>(2);
+    w.keys = A.take<uint64_t>(nt);
+    w.keys2 = A.take<uint64_t>(nt);
+    w.vals = A.take<int32_t>(nt);
+    w.par_i = A.take<int32_t>(ni);
+    w.par_l = A.take<int32_t>(nt);
+    w.child = A.take<int2>(ni);
+    w.nrange = A.take<int2>(ni);
+    w.llo = A.take<float4>(nt);
+    w.lhi = A.take<float4>(nt);
+    w.nlo = A.take<float4>(ni);
+    w.nhi = A.take<float4>(ni);
+    w.cost = A.take<float>(ni);
+    w.sort1 = A.take<char>((int64_t)sort1);
+    w.tl.visit = A.take<int>(ni);
+    w.tl.count = A.take<int>(ni);
+    w.tl.pos = A.take<int32_t>(nt);
+    w.tl.order2 = A.take<int32_t>(nt);
+    w.tl.par_l2 = A.take<int32_t>(nt);
+    w.tl.llo2 = A.take<float4>(nt);
+    w.tl.lhi2 = A.take<float4>(nt);
+    w.wide.items[0] = A.take<int2>(nt);
+    w.wide.items[1] = A.take<int2>(nt);
+    w.wide.counters = A.take<unsigned>(kWideCounters);
+    A.at = phase;
+    w.fn = A.take<float4>(nt);
+    w.vpn = A.take<float>(3 * nv);
+    w.ek = A.take<uint64_t>(3 * nt);
+    w.ek2 = A.take<uint64_t>(3 * nt);
+    w.ev = A.take<int32_t>(3 * nt);
+    w.ev2 = A.take<int32_t>(3 * nt);
+    w.en = A.take<float4>(3 * nt);
+    w.sort2 = A.take<char>((int64_t)sort2);
+}
 
+rt_status build(const float* V, int64_t nv, const int32_t* F, int64_t nt, cudaStream_t s, rt_scene* sc, const Work& w,
+                size_t sort1, size_t sort2)
+{
     {
-        DevBuf range;
-        ALLOC(range, 2 * sizeof(int));
         int r0[2] = {INT32_MAX, INT32_MIN}, r1[2];
-        RT_CUDA_TRY(cudaMemcpyAsync(range.p, r0, sizeof(r0), cudaMemcpyHostToDevice, s));
-        k_index_range<<<1024, kBlock, 0, s>>>(F, 3 * nt, range.as<int>());
+        RT_CUDA_TRY(cudaMemcpyAsync(w.range, r0, sizeof(r0), cudaMemcpyHostToDevice, s));
+        k_index_range<<<1024, kBlock, 0, s>>>(F, 3 * nt, w.range);
         RT_CUDA_TRY(cudaGetLastError());
-        RT_CUDA_TRY(cudaMemcpyAsync(r1, range.p, sizeof(r1), cudaMemcpyDeviceToHost, s));
+        RT_CUDA_TRY(cudaMemcpyAsync(r1, w.range, sizeof(r1), cudaMemcpyDeviceToHost, s));
         RT_CUDA_TRY(cudaStreamSynchronize(s));
         if (r1[0] < 0 || (int64_t)r1[1] >= nv)
             return rt_fail(RT_ERR_INVALID_ARG, "triangle vertex indices span [%d, %d], need [0, %lld)", r1[0], r1[1],
@@ -376,49 +419,37 @@ rt_status rt_build_scene(const float* V, int64_t nv, const int32_t* F, int64_t n
     }
     int init[12];
     for (int k = 0; k < 12; ++k) init[k] = (k % 6) < 3 ? INT32_MAX : INT32_MIN;
-    RT_CUDA_TRY(cudaMemcpyAsync(bounds.p, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    k_tri_bounds<<<grid_for(nt), kBlock, 0, s>>>(V, F, nt, cen.as<float4>(), bounds.as<int>());
+    RT_CUDA_TRY(cudaMemcpyAsync(w.bounds, init, sizeof(init), cudaMemcpyHostToDevice, s));
+    k_tri_bounds<<<grid_for(nt), kBlock, 0, s>>>(V, F, nt, w.cen, w.bounds);
     RT_CUDA_TRY(cudaGetLastError());
-    k_morton<<<grid_for(nt), kBlock, 0, s>>>(cen.as<float4>(), nt, bounds.as<int>(), keys.as<uint64_t>(),
-                                             vals.as<int32_t>());
+    k_morton<<<grid_for(nt), kBlock, 0, s>>>(w.cen, nt, w.bounds, w.keys, w.vals);
     RT_CUDA_TRY(cudaGetLastError());
+    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(w.sort1, sort1, w.keys, w.keys2, w.vals, w.order, (int)nt, 0, 64, s));
 
-    size_t tmp_bytes = 0;
-    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp_bytes, keys.as<uint64_t>(), keys2.as<uint64_t>(),
-                                                vals.as<int32_t>(), vals2.as<int32_t>(), (int)nt, 0, 64, s));
-    ALLOC(tmp, tmp_bytes);
-    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmp.p, tmp_bytes, keys.as<uint64_t>(), keys2.as<uint64_t>(),
-                                                vals.as<int32_t>(), vals2.as<int32_t>(), (int)nt, 0, 64, s));
-    const uint64_t* skeys = keys2.as<uint64_t>();
-    int32_t* order = vals2.as<int32_t>();
-
-    RT_CUDA_TRY(cudaMemsetAsync(visit.p, 0, (nt > 1 ? nt - 1 : 1) * sizeof(int), s));
-    RT_CUDA_TRY(cudaMemsetAsync(depth.p, 0, sizeof(int), s));
+    RT_CUDA_TRY(cudaMemsetAsync(w.tl.visit, 0, (nt > 1 ? nt - 1 : 1) * sizeof(int), s));
+    RT_CUDA_TRY(cudaMemsetAsync(w.depth, 0, sizeof(int), s));
     if (nt > 1) {
-        k_hierarchy<<<grid_for(nt - 1), kBlock, 0, s>>>(skeys, nt, child.as<int2>(), nrange.as<int2>(), par_i.as<int32_t>(),
-                                                        par_l.as<int32_t>());
+        k_hierarchy<<<grid_for(nt - 1), kBlock, 0, s>>>(w.keys2, nt, w.child, w.nrange, w.par_i, w.par_l);
         RT_CUDA_TRY(cudaGetLastError());
     } else {
         int m1 = -1;
-        RT_CUDA_TRY(cudaMemcpyAsync(par_l.p, &m1, sizeof(int), cudaMemcpyHostToDevice, s));
+        RT_CUDA_TRY(cudaMemcpyAsync(w.par_l, &m1, sizeof(int), cudaMemcpyHostToDevice, s));
     }
-    k_refit<<<grid_for(nt), kBlock, 0, s>>>(V, F, order, nt, child.as<int2>(), par_i.as<int32_t>(),
-                                            par_l.as<int32_t>(), llo.as<float4>(), lhi.as<float4>(),
-                                            nlo.as<float4>(), nhi.as<float4>(), visit.as<int>());
+    k_refit<<<grid_for(nt), kBlock, 0, s>>>(V, F, w.order, nt, w.child, w.par_i, w.par_l, w.llo, w.lhi, w.nlo, w.nhi, w.cost,
+                                            w.tl.visit);
     RT_CUDA_TRY(cudaGetLastError());
     if (nt > 2) {
-        rt_status ts = rt_treelet_optimise(nt, kTreeletPasses, child.as<int2>(), nrange.as<int2>(), par_i.as<int32_t>(),
-                                           par_l.as<int32_t>(), order, llo.as<float4>(), lhi.as<float4>(),
-                                           nlo.as<float4>(), nhi.as<float4>(), s);
+        rt_status ts = rt_treelet_optimise(nt, kTreeletPasses, w.child, w.nrange, w.par_i, w.par_l, w.order, w.llo, w.lhi,
+                                           w.nlo, w.nhi, w.cost, w.tl, s);
         if (ts != RT_OK) return ts;
     }
-    k_depth<<<grid_for(nt), kBlock, 0, s>>>(par_i.as<int32_t>(), par_l.as<int32_t>(), nt, depth.as<int>());
+    k_depth<<<grid_for(nt), kBlock, 0, s>>>(w.par_i, w.par_l, nt, w.depth);
     RT_CUDA_TRY(cudaGetLastError());
 
     int hb[12];
     int hdepth = 0;
-    RT_CUDA_TRY(cudaMemcpyAsync(hb, bounds.p, sizeof(hb), cudaMemcpyDeviceToHost, s));
-    RT_CUDA_TRY(cudaMemcpyAsync(&hdepth, depth.p, sizeof(int), cudaMemcpyDeviceToHost, s));
+    RT_CUDA_TRY(cudaMemcpyAsync(hb, w.bounds, sizeof(hb), cudaMemcpyDeviceToHost, s));
+    RT_CUDA_TRY(cudaMemcpyAsync(&hdepth, w.depth, sizeof(int), cudaMemcpyDeviceToHost, s));
     RT_CUDA_TRY(cudaStreamSynchronize(s));
     float mag = 0.f;
     for (int k = 0; k < 6; ++k) {
@@ -433,49 +464,75 @@ rt_status rt_build_scene(const float* V, int64_t nv, const int32_t* F, int64_t n
         return rt_fail(RT_ERR_DEVICE_LIMIT, "BVH depth %d exceeds the traversal stack (%d)", hdepth, RT_STACK_DEPTH);
     const float pad = ldexpf(mag, -18);
 
-    RT_CUDA_TRY(cudaMalloc(&sc->nodes, (size_t)(nt > 1 ? nt - 1 : 1) * sizeof(BNode)));
-    RT_CUDA_TRY(cudaMalloc(&sc->tris, (size_t)nt * 3 * sizeof(float4)));
-    RT_CUDA_TRY(cudaMalloc(&sc->pn, (size_t)nt * 7 * sizeof(float4)));
-    RT_CUDA_TRY(cudaMalloc(&sc->slot, (size_t)nt * sizeof(int32_t)));
+    {
+        // the scene's arrays, in one allocation (counted first, then handed out)
+        BuildArena A;
+        for (int pass = 0; pass < 2; ++pass) {
+            A.at = 0;
+            sc->nodes = A.take<BNode>(nt - 1);
+            sc->tris = A.take<float4>(nt * 3);
+            sc->pn = A.take<float4>(nt * 7);
+            sc->slot = A.take<int32_t>(nt);
+            sc->wnodes = A.take<WNode>(nt);
+            sc->wtris = A.take<float4>(nt * 3);
+            if (pass == 0) {
+                RT_CUDA_TRY(cudaMalloc(&sc->block, A.size));
+                A.base = static_cast<char*>(sc->block);
+            }
+        }
+    }
     sc->bytes = (int64_t)((nt > 1 ? nt - 1 : 1) * sizeof(BNode) + nt * 3 * sizeof(float4) + nt * 7 * sizeof(float4) +
                           nt * sizeof(int32_t));
     if (nt > 1) {
-        k_pack_nodes<<<grid_for(nt - 1), kBlock, 0, s>>>(child.as<int2>(), nt - 1, llo.as<float4>(), lhi.as<float4>(),
-                                                          nlo.as<float4>(), nhi.as<float4>(), pad, sc->nodes);
+        k_pack_nodes<<<grid_for(nt - 1), kBlock, 0, s>>>(w.child, nt - 1, w.llo, w.lhi, w.nlo, w.nhi, pad, sc->nodes);
         RT_CUDA_TRY(cudaGetLastError());
     }
-    k_pack_tris<<<grid_for(nt), kBlock, 0, s>>>(V, F, order, nt, sc->tris, sc->slot);
+    k_pack_tris<<<grid_for(nt), kBlock, 0, s>>>(V, F, w.order, nt, sc->tris, sc->slot);
     RT_CUDA_TRY(cudaGetLastError());
-    {
-        rt_status ws = rt_build_wide(sc, child.as<int2>(), nrange.as<int2>(), nlo.as<float4>(), nhi.as<float4>(),
-                                     llo.as<float4>(), lhi.as<float4>(), pad, s);
-        if (ws != RT_OK) return ws;
-    }
+    rt_status ws = rt_build_wide(sc, w.child, w.nrange, w.nlo, w.nhi, w.llo, w.lhi, pad, w.wide, s);
+    if (ws != RT_OK) return ws;
 
-    // pseudonormals
-    ALLOC(fn, nt * sizeof(float4));
-    ALLOC(vpn, nv * 3 * sizeof(float));
-    ALLOC(ek, 3 * nt * sizeof(uint64_t));
-    ALLOC(ek2, 3 * nt * sizeof(uint64_t));
-    ALLOC(ev, 3 * nt * sizeof(int32_t));
-    ALLOC(ev2, 3 * nt * sizeof(int32_t));
-    ALLOC(en, 3 * nt * sizeof(float4));
-    RT_CUDA_TRY(cudaMemsetAsync(vpn.p, 0, nv * 3 * sizeof(float), s));
-    k_face_normals<<<grid_for(nt), kBlock, 0, s>>>(V, F, nt, fn.as<float4>(), vpn.as<float>(), ek.as<uint64_t>(),
-                                                   ev.as<int32_t>());
+    // pseudonormals (the trees' scratch is free now)
+    RT_CUDA_TRY(cudaMemsetAsync(w.vpn, 0, nv * 3 * sizeof(float), s));
+    k_face_normals<<<grid_for(nt), kBlock, 0, s>>>(V, F, nt, w.fn, w.vpn, w.ek, w.ev);
     RT_CUDA_TRY(cudaGetLastError());
-    size_t tmp2 = 0;
-    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, tmp2, ek.as<uint64_t>(), ek2.as<uint64_t>(), ev.as<int32_t>(),
-                                                ev2.as<int32_t>(), (int)(3 * nt), 0, 64, s));
-    DevBuf tmpb;
-    ALLOC(tmpb, tmp2);
-    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(tmpb.p, tmp2, ek.as<uint64_t>(), ek2.as<uint64_t>(), ev.as<int32_t>(),
-                                                ev2.as<int32_t>(), (int)(3 * nt), 0, 64, s));
-    k_edge_normals<<<grid_for(3 * nt), kBlock, 0, s>>>(ek2.as<uint64_t>(), ev2.as<int32_t>(), 3 * nt, fn.as<float4>(),
-                                                       en.as<float4>());
+    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(w.sort2, sort2, w.ek, w.ek2, w.ev, w.ev2, (int)(3 * nt), 0, 64, s));
+    k_edge_normals<<<grid_for(3 * nt), kBlock, 0, s>>>(w.ek2, w.ev2, 3 * nt, w.fn, w.en);
     RT_CUDA_TRY(cudaGetLastError());
-    k_pack_pn<<<grid_for(nt), kBlock, 0, s>>>(F, order, nt, fn.as<float4>(), en.as<float4>(), vpn.as<float>(), sc->pn);
+    k_pack_pn<<<grid_for(nt), kBlock, 0, s>>>(F, w.order, nt, w.fn, w.en, w.vpn, sc->pn);
     RT_CUDA_TRY(cudaGetLastError());
     RT_CUDA_TRY(cudaStreamSynchronize(s));
     return RT_OK;
+}
+
+}  // namespace
+
+rt_status rt_build_scene(const float* V, int64_t nv, const int32_t* F, int64_t nt, cudaStream_t s, rt_scene* sc)
+{
+    sc->n_tris = nt;
+    sc->n_verts = nv;
+    sc->n_nodes = nt - 1;
+    size_t sort1 = 0, sort2 = 0;
+    uint64_t* key = nullptr;
+    int32_t* val = nullptr;
+    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort1, key, key, val, val, (int)nt, 0, 64, s));
+    RT_CUDA_TRY(cub::DeviceRadixSort::SortPairs(nullptr, sort2, key, key, val, val, (int)(3 * nt), 0, 64, s));
+    BuildArena A;
+    Work w;
+    lay_out(A, w, nt, nv, sort1, sort2);
+    // Small scenes from the library's pool; a large one's scratch is given back, and
+    // an allocation of its own is then cheaper than a stream-ordered one (400 MB:
+    // 79 + 195 us against 350 + 590).
+    const bool pooled = A.size <= kScratchKept;
+    void* scratch = nullptr;
+    rt_status st = RT_OK;
+    if (pooled) st = rt_scratch_alloc(&scratch, A.size, s);
+    else RT_CUDA_TRY(cudaMalloc(&scratch, A.size));
+    if (st != RT_OK) return st;
+    A.base = static_cast<char*>(scratch);
+    lay_out(A, w, nt, nv, sort1, sort2);
+    st = build(V, nv, F, nt, s, sc, w, sort1, sort2);
+    const cudaError_t e = pooled ? cudaFreeAsync(scratch, s) : cudaFree(scratch);
+    if (st == RT_OK && e != cudaSuccess) st = rt_cuda_fail(e, "releasing the build's scratch");
+    return st;
 }

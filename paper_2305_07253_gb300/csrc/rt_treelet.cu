@@ -23,20 +23,12 @@ constexpr int kTreelet = 7;             // treelet leaves
 constexpr int kSubsets = 1 << kTreelet;
 constexpr int kGroup = 8;               // lanes that work on one treelet
 constexpr int kGroups = 32 / kGroup;    // treelets a warp works on at a time
-constexpr float kCostNode = 1.2f;       // surface-area cost of visiting a node ...
-constexpr float kCostTri = 1.0f;        // ... and of testing a triangle
+using rttree::half_area;
+using rttree::kCostNode;
+using rttree::kCostTri;
 constexpr int kMaxWalk = 256;
 
-// Half the surface area of a box, every rounding written out: the restructured
-// tree must not depend on how a compiler contracts these sums in one place or
-// another (an ulp decides between two topologies of nearly equal cost).
-__device__ __forceinline__ float half_area(float4 lo, float4 hi)
-{
-    const float dx = __fsub_rn(hi.x, lo.x), dy = __fsub_rn(hi.y, lo.y), dz = __fsub_rn(hi.z, lo.z);
-    return __fmaf_rn(dz, dx, __fmaf_rn(dx, dy, __fmul_rn(dy, dz)));
-}
-
-// the same for the subsets that the dynamic program compares
+// half the surface area of the subsets that the dynamic program compares (rounded as its sums always were)
 __device__ __forceinline__ float subset_half_area(float4 lo, float4 hi)
 {
     const float dx = __fsub_rn(hi.x, lo.x), dy = __fsub_rn(hi.y, lo.y), dz = __fsub_rn(hi.z, lo.z);
@@ -55,30 +47,6 @@ struct Tree {
     int* visit;
     int64_t n_leaves;
 };
-
-__device__ __forceinline__ float4 ref_lo(const Tree& T, int r) { return r < 0 ? __ldcg(T.llo + ~r) : __ldcg(T.nlo + r); }
-__device__ __forceinline__ float4 ref_hi(const Tree& T, int r) { return r < 0 ? __ldcg(T.lhi + ~r) : __ldcg(T.nhi + r); }
-__device__ __forceinline__ float ref_cost(const Tree& T, int r)
-{
-    return r < 0 ? kCostTri * half_area(ref_lo(T, r), ref_hi(T, r)) : __ldcg(T.cost + r);
-}
-
-// initial subtree costs, bottom-up
-__global__ void k_cost(Tree T)
-{
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= T.n_leaves) return;
-    int32_t node = T.par_l[k];
-    for (int guard = 0; node >= 0 && guard < kMaxWalk; ++guard) {
-        if (atomicAdd(&T.visit[node], 1) == 0) return;
-        __threadfence();
-        const int2 c = __ldcg(T.child + node);
-        T.cost[node] = __fadd_rn(__fmaf_rn(kCostNode, half_area(__ldcg(T.nlo + node), __ldcg(T.nhi + node)), ref_cost(T, c.x)),
-                                 ref_cost(T, c.y));
-        __threadfence();
-        node = T.par_i[node];
-    }
-}
 
 // One treelet's shared memory.  Its size is 32 bytes past a multiple of 128, so
 // that the four treelets of a warp start eight banks apart.
@@ -316,7 +284,7 @@ __device__ void optimise_treelets(const Tree& T, int root, Workspace& w, const u
             const int S = w.set[i], P = w.part[S];
             float4 lo2, hi2;
             subset_box(w, S, lo2, hi2);
-            w.copt[S] = __fadd_rn(__fmaf_rn(kCostNode, half_area(lo2, hi2), w.copt[P]), w.copt[S ^ P]);
+            w.copt[S] = rttree::node_cost(lo2, hi2, w.copt[P], w.copt[S ^ P]);
         }
     }
     __syncwarp();
@@ -337,9 +305,11 @@ __device__ void optimise_treelets(const Tree& T, int root, Workspace& w, const u
     __syncwarp();
 }
 
-// one restructuring pass: leaves walk up; each node whose second child finished
+// One restructuring pass: leaves walk up; each node whose second child finished
 // is optimised by the warp of the thread that finished it, four at a time.  A
-// node over two leaves has one topology only and is passed.
+// node over two leaves has one topology only and is passed.  (Passing, in later
+// passes, the nodes below and around which nothing had changed since they were
+// last looked at saved nothing: few are left out.)
 __global__ void __launch_bounds__(kBlock) k_treelets(Tree T)
 {
     __shared__ Workspace ws[kWarps * kGroups];
@@ -455,64 +425,28 @@ unsigned grid_for(int64_t n) { return (unsigned)((n + kBlock - 1) / kBlock); }
 }  // namespace
 
 rt_status rt_treelet_optimise(int64_t nt, int passes, int2* child, int2* range, int32_t* par_i, int32_t* par_l,
-                              int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, cudaStream_t s)
+                              int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, float* cost,
+                              const TreeletScratch& ws, cudaStream_t s)
 {
     if (nt < 3 || passes <= 0) return RT_OK;
     const int64_t ni = nt - 1;
-    float* cost = nullptr;
-    int* visit = nullptr;
-    int* count = nullptr;
-    int32_t* pos = nullptr;
-    int32_t* order2 = nullptr;
-    int32_t* par_l2 = nullptr;
-    float4* llo2 = nullptr;
-    float4* lhi2 = nullptr;
-    rt_status st = RT_OK;
-    cudaError_t e = cudaSuccess;
-#define TRY_ALLOC(p, bytes) \
-    if (e == cudaSuccess) e = cudaMallocAsync((void**)&(p), (size_t)(bytes), s)
-    TRY_ALLOC(cost, ni * sizeof(float));
-    TRY_ALLOC(visit, ni * sizeof(int));
-    TRY_ALLOC(count, ni * sizeof(int));
-    TRY_ALLOC(pos, nt * sizeof(int32_t));
-    TRY_ALLOC(order2, nt * sizeof(int32_t));
-    TRY_ALLOC(par_l2, nt * sizeof(int32_t));
-    TRY_ALLOC(llo2, nt * sizeof(float4));
-    TRY_ALLOC(lhi2, nt * sizeof(float4));
-#undef TRY_ALLOC
-    if (e != cudaSuccess) st = rt_cuda_fail(e, "cudaMallocAsync");
-    Tree T = {child, par_i, par_l, llo, lhi, nlo, nhi, cost, visit, nt};
-    if (st == RT_OK) {
-        e = cudaMemsetAsync(visit, 0, ni * sizeof(int), s);
-        if (e == cudaSuccess) k_cost<<<grid_for(nt), kBlock, 0, s>>>(T);
-        for (int pass = 0; pass < passes && e == cudaSuccess; ++pass) {
-            e = cudaMemsetAsync(visit, 0, ni * sizeof(int), s);
-            if (e == cudaSuccess) k_treelets<<<grid_for(nt), kBlock, 0, s>>>(T);
-        }
-        // depth-first leaf order
-        if (e == cudaSuccess) e = cudaMemsetAsync(visit, 0, ni * sizeof(int), s);
-        if (e == cudaSuccess) {
-            k_counts<<<grid_for(nt), kBlock, 0, s>>>(child, par_i, par_l, nt, count, visit);
-            k_leaf_position<<<grid_for(nt), kBlock, 0, s>>>(child, par_i, par_l, count, nt, pos);
-            k_node_range<<<grid_for(ni), kBlock, 0, s>>>(child, par_i, count, ni, range);
-            k_permute_leaves<<<grid_for(nt), kBlock, 0, s>>>(pos, nt, order, llo, lhi, order2, llo2, lhi2, par_l2,
-                                                             par_l);
-            k_remap_children<<<grid_for(ni), kBlock, 0, s>>>(child, ni, pos);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(order, order2, nt * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(par_l, par_l2, nt * sizeof(int32_t), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(llo, llo2, nt * sizeof(float4), cudaMemcpyDeviceToDevice, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(lhi, lhi2, nt * sizeof(float4), cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) st = rt_cuda_fail(e, "treelet restructuring");
+    const Tree T = {child, par_i, par_l, llo, lhi, nlo, nhi, cost, ws.visit, nt};
+    for (int pass = 0; pass < passes; ++pass) {
+        RT_CUDA_TRY(cudaMemsetAsync(ws.visit, 0, ni * sizeof(int), s));
+        k_treelets<<<grid_for(nt), kBlock, 0, s>>>(T);
     }
-    cudaFreeAsync(cost, s);
-    cudaFreeAsync(visit, s);
-    cudaFreeAsync(count, s);
-    cudaFreeAsync(pos, s);
-    cudaFreeAsync(order2, s);
-    cudaFreeAsync(par_l2, s);
-    cudaFreeAsync(llo2, s);
-    cudaFreeAsync(lhi2, s);
-    return st;
+    // depth-first leaf order
+    RT_CUDA_TRY(cudaMemsetAsync(ws.visit, 0, ni * sizeof(int), s));
+    k_counts<<<grid_for(nt), kBlock, 0, s>>>(child, par_i, par_l, nt, ws.count, ws.visit);
+    k_leaf_position<<<grid_for(nt), kBlock, 0, s>>>(child, par_i, par_l, ws.count, nt, ws.pos);
+    k_node_range<<<grid_for(ni), kBlock, 0, s>>>(child, par_i, ws.count, ni, range);
+    k_permute_leaves<<<grid_for(nt), kBlock, 0, s>>>(ws.pos, nt, order, llo, lhi, ws.order2, ws.llo2, ws.lhi2, ws.par_l2,
+                                                     par_l);
+    k_remap_children<<<grid_for(ni), kBlock, 0, s>>>(child, ni, ws.pos);
+    RT_CUDA_TRY(cudaGetLastError());
+    RT_CUDA_TRY(cudaMemcpyAsync(order, ws.order2, nt * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    RT_CUDA_TRY(cudaMemcpyAsync(par_l, ws.par_l2, nt * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    RT_CUDA_TRY(cudaMemcpyAsync(llo, ws.llo2, nt * sizeof(float4), cudaMemcpyDeviceToDevice, s));
+    RT_CUDA_TRY(cudaMemcpyAsync(lhi, ws.lhi2, nt * sizeof(float4), cudaMemcpyDeviceToDevice, s));
+    return RT_OK;
 }

@@ -29,10 +29,8 @@ struct Entry {
     float lo[3], hi[3];
 };
 
-struct Item {
-    int bin;   // binary internal node, or ~triangle for a one-triangle scene
-    int slot;  // wide node index to write
-};
+// An item is a binary internal node (or ~triangle for a one-triangle scene) and
+// the wide node index to write.
 
 __device__ __forceinline__ void entry_of(int c, const int2* range, const float4* nlo, const float4* nhi,
                                          const float4* llo, const float4* lhi, Entry& e)
@@ -63,24 +61,21 @@ __device__ __forceinline__ float half_area(const Entry& e)
     return dx * dy + dy * dz + dz * dx;
 }
 
-__global__ void k_collapse(const Item* items, unsigned n_items, const int2* child, const int2* range,
+__device__ __forceinline__ void collapse_item(const int2 item, const int2* child, const int2* range,
                            const float4* nlo, const float4* nhi, const float4* llo, const float4* lhi,
-                           const float4* tris, float pad, Item* next, unsigned* next_count, unsigned* node_counter,
+                           const float4* tris, float pad, int2* next, unsigned* next_count, unsigned* node_counter,
                            unsigned* tri_counter, WNode* wn, float4* wtris, unsigned max_nodes, unsigned n_tris,
                            int* error)
 {
-    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_items) return;
-    const Item it = items[i];
     Entry E[8];
     int ne = 0;
-    if (it.bin >= 0) {
-        const int2 c = child[it.bin];
+    if (item.x >= 0) {
+        const int2 c = child[item.x];
         entry_of(c.x, range, nlo, nhi, llo, lhi, E[0]);
         entry_of(c.y, range, nlo, nhi, llo, lhi, E[1]);
         ne = 2;
     } else {
-        entry_of(it.bin, range, nlo, nhi, llo, lhi, E[0]);
+        entry_of(item.x, range, nlo, nhi, llo, lhi, E[0]);
         ne = 1;
     }
     // open the largest inner child until 8 children
@@ -198,8 +193,7 @@ __global__ void k_collapse(const Item* items, unsigned n_items, const int2* chil
             const int s = slot_of[j];
             const unsigned w = cb + __popc(imask & ((1u << s) - 1u));
             const unsigned k = atomicAdd(next_count, 1u);
-            next[k].bin = E[j].ref;
-            next[k].slot = (int)w;
+            next[k] = make_int2(E[j].ref, (int)w);
         }
     auto pack4 = [](const unsigned char* b) {
         return (unsigned)b[0] | ((unsigned)b[1] << 8) | ((unsigned)b[2] << 16) | ((unsigned)b[3] << 24);
@@ -210,57 +204,70 @@ __global__ void k_collapse(const Item* items, unsigned n_items, const int2* chil
     n.q0 = make_uint4(pack4(qlo[0]), pack4(qlo[0] + 4), pack4(qlo[1]), pack4(qlo[1] + 4));
     n.q1 = make_uint4(pack4(qlo[2]), pack4(qlo[2] + 4), pack4(qhi[0]), pack4(qhi[0] + 4));
     n.q2 = make_uint4(pack4(qhi[1]), pack4(qhi[1] + 4), pack4(qhi[2]), pack4(qhi[2] + 4));
-    wn[it.slot] = n;
+    wn[item.y] = n;
 }
 
-struct Buf {
-    void* p = nullptr;
-    ~Buf() { if (p) cudaFree(p); }
-};
+__global__ void k_collapse(const int2* items, const unsigned* n_items, const int2* child, const int2* range,
+                           const float4* nlo, const float4* nhi, const float4* llo, const float4* lhi,
+                           const float4* tris, float pad, int2* next, unsigned* next_count, unsigned* node_counter,
+                           unsigned* tri_counter, WNode* wn, float4* wtris, unsigned max_nodes, unsigned n_tris,
+                           int* error)
+{
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < *n_items; i += gridDim.x * blockDim.x)
+        collapse_item(items[i], child, range, nlo, nhi, llo, lhi, tris, pad, next, next_count, node_counter, tri_counter, wn, wtris, max_nodes, n_tris, error);
+}
 
 }  // namespace
 
 rt_status rt_build_wide(rt_scene* sc, const int2* child, const int2* range, const float4* node_lo,
                         const float4* node_hi, const float4* leaf_lo, const float4* leaf_hi, float pad,
-                        cudaStream_t s)
+                        const WideScratch& ws, cudaStream_t s)
 {
     const int64_t nt = sc->n_tris;
     const unsigned max_nodes = (unsigned)(nt > 1 ? nt : 1);
-    RT_CUDA_TRY(cudaMalloc(&sc->wnodes, (size_t)max_nodes * sizeof(WNode)));
-    RT_CUDA_TRY(cudaMalloc(&sc->wtris, (size_t)nt * 3 * sizeof(float4)));
-    Buf items[2], ctr;
-    RT_CUDA_TRY(cudaMalloc(&items[0].p, (size_t)max_nodes * sizeof(Item)));
-    RT_CUDA_TRY(cudaMalloc(&items[1].p, (size_t)max_nodes * sizeof(Item)));
-    RT_CUDA_TRY(cudaMalloc(&ctr.p, 4 * sizeof(unsigned)));
-    unsigned* c = static_cast<unsigned*>(ctr.p);  // [0] nodes, [1] triangles, [2] next count, [3] error
-    const unsigned init[4] = {1u, 0u, 0u, 0u};
+    unsigned* c = ws.counters;  // [0] nodes, [1] triangles, [2] error; [4 + l] items of level l
+    const int2 root = make_int2(nt > 1 ? 0 : ~0, 0);
+    unsigned init[kWideCounters] = {1u};
+    init[4] = 1u;
     RT_CUDA_TRY(cudaMemcpyAsync(c, init, sizeof(init), cudaMemcpyHostToDevice, s));
-    Item root = {nt > 1 ? 0 : ~0, 0};
-    RT_CUDA_TRY(cudaMemcpyAsync(items[0].p, &root, sizeof(Item), cudaMemcpyHostToDevice, s));
-    unsigned n_items = 1;
+    RT_CUDA_TRY(cudaMemcpyAsync(ws.items[0], &root, sizeof(root), cudaMemcpyHostToDevice, s));
+    int dev = 0, sms = 0;
+    RT_CUDA_TRY(cudaGetDevice(&dev));
+    RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // Levels are launched without knowing how many there are: as many as a scene of
+    // this size mostly has, then a look at the counts, then more if items are left
+    // (a synchronisation per level cost as much as the small levels themselves).
+    int ahead = 4;
+    for (int64_t t = nt; t > 1; t >>= 2) ++ahead;
     int level = 0;
-    for (; n_items > 0; ++level) {
-        if (level > 256) return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH collapse did not terminate");
-        RT_CUDA_TRY(cudaMemsetAsync(c + 2, 0, sizeof(unsigned), s));
-        k_collapse<<<(n_items + kBlock - 1) / kBlock, kBlock, 0, s>>>(
-            static_cast<const Item*>(items[level & 1].p), n_items, child, range, node_lo, node_hi, leaf_lo, leaf_hi,
-            sc->tris, pad, static_cast<Item*>(items[(level + 1) & 1].p), c + 2, c, c + 1, sc->wnodes, sc->wtris,
-            max_nodes, (unsigned)nt, reinterpret_cast<int*>(c + 3));
+    unsigned h[kWideCounters];
+    for (;;) {
+        const int stop = level + ahead < 256 ? level + ahead : 256;
+        for (; level < stop; ++level) {
+            // a level has at most 8^level items
+            const int64_t most = level < 8 ? (int64_t)1 << (3 * level) : max_nodes;
+            int64_t blocks = ((most < max_nodes ? most : max_nodes) + kBlock - 1) / kBlock;
+            if (blocks > 16 * (int64_t)sms) blocks = 16 * (int64_t)sms;
+            k_collapse<<<(unsigned)blocks, kBlock, 0, s>>>(ws.items[level & 1], c + 4 + level, child, range, node_lo, node_hi,
+                                                           leaf_lo, leaf_hi, sc->tris, pad, ws.items[(level + 1) & 1],
+                                                           c + 5 + level, c, c + 1, sc->wnodes, sc->wtris, max_nodes,
+                                                           (unsigned)nt, reinterpret_cast<int*>(c + 2));
+        }
         RT_CUDA_TRY(cudaGetLastError());
-        unsigned h[4];
         RT_CUDA_TRY(cudaMemcpyAsync(h, c, sizeof(h), cudaMemcpyDeviceToHost, s));
         RT_CUDA_TRY(cudaStreamSynchronize(s));
-        if (h[3]) return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH collapse ran out of node or triangle slots");
-        n_items = h[2];
-        sc->n_wnodes = h[0];
-        if (n_items == 0 && h[1] != (unsigned)nt)
-            return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH holds %u of %lld triangles", h[1], (long long)nt);
+        if (h[2]) return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH collapse ran out of node or triangle slots");
+        if (h[4 + level] == 0) break;
+        if (level >= 256) return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH collapse did not terminate");
+        ahead = 8;
     }
+    if (h[1] != (unsigned)nt)
+        return rt_fail(RT_ERR_DEVICE_LIMIT, "wide BVH holds %u of %lld triangles", h[1], (long long)nt);
+    sc->n_wnodes = h[0];
+    while (level > 0 && h[4 + level - 1] == 0) --level;  // the levels that had items
     sc->wide_depth = level;
     sc->bytes += (int64_t)sc->n_wnodes * (int64_t)sizeof(WNode) + nt * 3 * (int64_t)sizeof(float4);
-    if (level > RT_WSTACK_DEPTH) {  // deeper than the traversal stack: keep the binary tree only
-        cudaFree(sc->wnodes);
-        cudaFree(sc->wtris);
+    if (level > RT_WSTACK_DEPTH) {  // deeper than the traversal stack: the binary tree only
         sc->wnodes = nullptr;
         sc->wtris = nullptr;
     }
