@@ -88,50 +88,48 @@ __device__ __forceinline__ float tri_d2_rn(const float* p, const float* a, const
     return dot3r(pq, pq);
 }
 
-__device__ __forceinline__ bool axis_separates(const float* ax, const float* v0, const float* v1, const float* v2,
-                                               const float* hs)
+// Separation along an axis on which the triangle's vertices lie at p0, p1, p2 and
+// the box reaches r to either side of the origin
+__device__ __forceinline__ bool separated(float p0, float p1, float p2, float r)
 {
-    const float p0 = dot3r(ax, v0), p1 = dot3r(ax, v1), p2 = dot3r(ax, v2);
-    const float lo = fminf(fminf(p0, p1), p2), hi = fmaxf(fmaxf(p0, p1), p2);
-    const float r = __fadd_rn(__fadd_rn(__fmul_rn(hs[0], fabsf(ax[0])), __fmul_rn(hs[1], fabsf(ax[1]))),
-                              __fmul_rn(hs[2], fabsf(ax[2])));
-    return lo > r || hi < -r;
+    return rtdev::min3f(p0, p1, p2) > r || rtdev::max3f(p0, p1, p2) < -r;
 }
 
-// triangle / box overlap by separating axes (touching counts)
+// Triangle / box overlap by separating axes (touching counts).  Components of an
+// axis that are zero are left out: adding their products changes nothing.
 __device__ bool tri_box(const float* c, const float* hs, const float* A, const float* B, const float* C)
 {
-    float v0[3], v1[3], v2[3], e[3][3];
+    float v[3][3], e[3][3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        v0[k] = __fsub_rn(A[k], c[k]);
-        v1[k] = __fsub_rn(B[k], c[k]);
-        v2[k] = __fsub_rn(C[k], c[k]);
+        v[0][k] = __fsub_rn(A[k], c[k]);
+        v[1][k] = __fsub_rn(B[k], c[k]);
+        v[2][k] = __fsub_rn(C[k], c[k]);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        e[0][k] = __fsub_rn(v1[k], v0[k]);
-        e[1][k] = __fsub_rn(v2[k], v1[k]);
-        e[2][k] = __fsub_rn(v0[k], v2[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        float ax[3] = {0.f, 0.f, 0.f};
-        ax[k] = 1.f;
-        if (axis_separates(ax, v0, v1, v2, hs)) return false;
+        if (separated(v[0][k], v[1][k], v[2][k], hs[k])) return false;
+        e[0][k] = __fsub_rn(v[1][k], v[0][k]);
+        e[1][k] = __fsub_rn(v[2][k], v[1][k]);
+        e[2][k] = __fsub_rn(v[0][k], v[2][k]);
     }
     const float n[3] = {__fsub_rn(__fmul_rn(e[0][1], e[1][2]), __fmul_rn(e[0][2], e[1][1])),
                         __fsub_rn(__fmul_rn(e[0][2], e[1][0]), __fmul_rn(e[0][0], e[1][2])),
                         __fsub_rn(__fmul_rn(e[0][0], e[1][1]), __fmul_rn(e[0][1], e[1][0]))};
-    if (axis_separates(n, v0, v1, v2, hs)) return false;
+    const float an[3] = {fabsf(n[0]), fabsf(n[1]), fabsf(n[2])};
+    if (separated(dot3r(n, v[0]), dot3r(n, v[1]), dot3r(n, v[2]), dot3r(hs, an))) return false;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const float ax0[3] = {0.f, -e[j][2], e[j][1]};
-        const float ax1[3] = {e[j][2], 0.f, -e[j][0]};
-        const float ax2[3] = {-e[j][1], e[j][0], 0.f};
-        if (axis_separates(ax0, v0, v1, v2, hs) || axis_separates(ax1, v0, v1, v2, hs) ||
-            axis_separates(ax2, v0, v1, v2, hs))
-            return false;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            // unit axis k x edge j: (0, -e2, e1), (e2, 0, -e0), (-e1, e0, 0), its two
+            // components in the order of the coordinates
+            const int s = k == 0 ? 1 : 0, t = k == 2 ? 1 : 2;
+            const float es = k == 1 ? e[j][t] : -e[j][t], et = k == 1 ? -e[j][s] : e[j][s];
+            auto on = [&](const float* q) { return __fadd_rn(__fmul_rn(es, q[s]), __fmul_rn(et, q[t])); };
+            const float r = __fadd_rn(__fmul_rn(hs[s], fabsf(es)), __fmul_rn(hs[t], fabsf(et)));
+            if (separated(on(v[0]), on(v[1]), on(v[2]), r)) return false;
+        }
     }
     return true;
 }
