@@ -253,6 +253,7 @@ rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 // resident at once (rt_launch_trace has the figures)
 constexpr int64_t kSmallCall = 131072;
 constexpr int64_t kSmallCallTriangles = 65536;  // calls that trace triangles only
+constexpr int kSmallBlock = 128;                // their threads per block, whatever the tuning's
 
 // conc_set: the set of library streams a concurrent program of this call uses
 rt_status rt_launch_trace(const TraceArgs& a, bool counted, cudaStream_t s, StageTiming* timing = nullptr,

@@ -753,7 +753,10 @@ rt_status rt_launch_trace(const TraceArgs& a0, bool counted, cudaStream_t s, Sta
     if (wavefront)
         return counted ? run_wavefront<true>(a, tu, s, timing, conc_set)
                        : run_wavefront<false>(a, tu, s, timing, conc_set);
-    const int64_t blocks = (a.n + tu.block - 1) / tu.block;
+    // the tuning's block where it selects this kernel; a small call's own otherwise
+    // (the stage kernels hold larger blocks than this one's registers allow)
+    const int block = tu.kernel == RT_KERNEL_SIMPLE ? tu.block : kSmallBlock;
+    const int64_t blocks = (a.n + block - 1) / block;
     if (blocks > 0x7fffffffLL) return rt_fail(RT_ERR_INVALID_ARG, "too many rays");
     Marks marks{timing};
     if (timing) timing->n_launches = 0;
@@ -782,11 +785,11 @@ rt_status rt_launch_trace(const TraceArgs& a0, bool counted, cudaStream_t s, Sta
         const unsigned nb = (unsigned)blocks;
         const int L = grid_layout_of(a);
         if (a.wnodes) {
-            if (counted) launch_simple<true, true>(a, L, nb, tu.block, s);
-            else launch_simple<false, true>(a, L, nb, tu.block, s);
+            if (counted) launch_simple<true, true>(a, L, nb, block, s);
+            else launch_simple<false, true>(a, L, nb, block, s);
         } else {
-            if (counted) launch_simple<true, false>(a, L, nb, tu.block, s);
-            else launch_simple<false, false>(a, L, nb, tu.block, s);
+            if (counted) launch_simple<true, false>(a, L, nb, block, s);
+            else launch_simple<false, false>(a, L, nb, block, s);
         }
         e = cudaGetLastError();
         if (e == cudaSuccess) st = marks.end(s);

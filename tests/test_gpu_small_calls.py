@@ -98,3 +98,18 @@ def test_capture(world):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(hits, want) and torch.equal(other, want)
+
+
+@pytest.mark.parametrize("block", [32, 1024])
+def test_any_block_of_the_tuning(world, block):
+    """A block that only the stage kernels can hold still serves small calls."""
+    rq, scene, fields, rays = world
+    p = rq.split_params(mode=1, m_near=2.0)
+    want = rq.rt_trace_combined(scene, fields[0], rays[:777], p)
+    prev = rq.rt_set_tuning(block=block)
+    try:
+        got = rq.rt_trace_combined(scene, fields[0], rays[:777], p)
+        batch = rq.rt_trace_batches(scene, fields[0], [(rays[:777], p)])[0]
+    finally:
+        rq.rt_set_tuning(prev)
+    assert torch.equal(got, want) and torch.equal(batch, want)
