@@ -391,8 +391,10 @@ __device__ __forceinline__ int64_t sample_index(const BakeArgs& b, const int32_t
     return ii[0] + (int64_t)b.n[0] * (ii[1] + (int64_t)b.n[1] * ii[2]);
 }
 
+// 16 blocks (32 warps) an SM, 64 registers: 256^3 10.95 ms; the compiler's own 72
+// registers 11.32, 18 blocks 11.07, 20 blocks (with spills) 12.02.
 template <int LS>
-__global__ void __launch_bounds__(32 * kBrickWarps) k_bake_bricks(const BakeArgs b, const PacketGrid pg)
+__global__ void __launch_bounds__(32 * kBrickWarps, 16) k_bake_bricks(const BakeArgs b, const PacketGrid pg)
 {
     constexpr int S = 1 << LS;
     __shared__ BrickShared shared[kBrickWarps];
