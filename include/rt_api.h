@@ -250,7 +250,7 @@ rt_status rt_sdf_sites(const rt_scene* scene, const rt_sdf* sdf, int32_t stage, 
  * that level's voxel instead of the grid's smallest voxel edge; t_1 uses
  * the voxel at the query's start point o + t_min d and t_2 the voxel at its end
  * point o + t_max d (Section 3, "GI & Shadow Rays"); the march is clipped to
- * the coarsest level's box.  A cascade is always read through its cell-corner
+ * the coarsest level's box.  A cascade is always read through its cell
  * copy: fill it with rt_sdf_bake (or write the values and call rt_sdf_prepare)
  * before tracing; a trace before that returns RT_ERR_INVALID_ARG, as does
  * rt_trace_combined_backward on a cascade.  Errors: RT_ERR_INVALID_ARG for
