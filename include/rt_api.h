@@ -178,7 +178,8 @@ rt_status rt_sdf_destroy(rt_sdf* sdf);
  * after an optimiser step), otherwise the traces keep reading the old copy.
  * Traces read the plain grid until the first prepare, or when the tuning
  * selects the plain layout.  Also builds the x-pair copy (see rt_tuning).
- * Memory: about 4x (cells) + 2x (pairs) the grid, owned by the handle,
+ * A float32 grid of 2^26 faces or more keeps both faces of every cell together.
+ * Memory: about 4x (cells; such a grid 8x) + 2x (pairs) the grid, owned by the handle,
  * released by rt_sdf_destroy.  On a cascade: the cell copy of every level
  * (no x-pair copy).  Enqueued on `stream`. */
 rt_status rt_sdf_prepare(rt_sdf* sdf, void* stream);

@@ -125,6 +125,10 @@ rt_status rt_fill_trace_args(TraceArgs& a, const rt_scene* sc, const rt_sdf* sdf
         a.cells = sdf->cells;
         a.pairs = sdf->pairs;
         a.grid_f16 = sdf->dtype == RT_GRID_F16;
+        if (sdf->levels == 0) {
+            a.cell_step = (a.grid_f16 ? 8 : 16) << rtdev::cell_shift(rtdev::cell_count(sdf->n[0], sdf->n[1], sdf->n[2]), a.grid_f16);
+            a.cell_row = (int64_t)a.cell_step * sdf->n[0];
+        }
         for (int k = 0; k < 3; ++k) {
             a.glo[k] = sdf->lo[k];
             a.ghi[k] = sdf->hi[k];

@@ -477,8 +477,8 @@ __device__ __forceinline__ Quad<float2> quad(float a, float b, float c, float d)
 
 template <class T, class V2, class V4>
 __global__ void __launch_bounds__(kCopyBlock) k_copies(const T* __restrict__ grid, int32_t nx, int32_t ny, int32_t nz,
-                                                       int64_t samples, int64_t entries, V4* __restrict__ cells,
-                                                       V2* __restrict__ pairs)
+                                                       int64_t samples, int64_t entries, int shift,
+                                                       V4* __restrict__ cells, V2* __restrict__ pairs)
 {
     static_assert(sizeof(V4) == sizeof(Quad<V2>), "one entry is two pairs");
     const uint32_t chunks = (uint32_t)((nx + kCopyBlock - 1) / kCopyBlock);
@@ -498,23 +498,25 @@ __global__ void __launch_bounds__(kCopyBlock) k_copies(const T* __restrict__ gri
         }
         if (j + 1 < ny && k + 1 < nz) {
             const Quad<V2> q = quad(v, g[nx], g[(int64_t)nx * ny], g[(int64_t)nx * ny + nx]);
-            cells[blockIdx.y * entries + i + (int64_t)nx * (j + (int64_t)(ny - 1) * k)] = *reinterpret_cast<const V4*>(&q);
+            const int64_t e = (blockIdx.y * entries + rtdev::cell_slot(i, j, k, nx, ny)) << shift;
+            cells[e] = *reinterpret_cast<const V4*>(&q);
+            if (shift && i > 0) cells[e - 1] = *reinterpret_cast<const V4*>(&q);
         }
     }
 }
 
 // `levels` grids one after another from `grid` (pairs only for one)
-rt_status launch_copies(const void* grid, int32_t dtype, const int32_t n[3], int levels, void* cells, void* pairs,
-                        cudaStream_t s)
+rt_status launch_copies(const void* grid, int32_t dtype, const int32_t n[3], int levels, int shift, void* cells,
+                        void* pairs, cudaStream_t s)
 {
     const int64_t total = (int64_t)((n[0] + kCopyBlock - 1) / kCopyBlock) * n[1] * n[2];
     const dim3 blocks((unsigned)(total < 0x7fffffffLL ? total : 0x7fffffffLL), (unsigned)levels);
     const int64_t samples = (int64_t)n[0] * n[1] * n[2], entries = rtdev::cell_count(n[0], n[1], n[2]);
     if (dtype == RT_GRID_F16)
-        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const __half*>(grid), n[0], n[1], n[2], samples, entries,
+        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const __half*>(grid), n[0], n[1], n[2], samples, entries, shift,
                                                static_cast<uint2*>(cells), static_cast<__half2*>(pairs));
     else
-        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const float*>(grid), n[0], n[1], n[2], samples, entries,
+        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const float*>(grid), n[0], n[1], n[2], samples, entries, shift,
                                                static_cast<float4*>(cells), static_cast<float2*>(pairs));
     RT_CUDA_TRY(cudaGetLastError());
     return RT_OK;
@@ -540,20 +542,21 @@ rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int first, int count, cudaS
     const int64_t n = sdf->n[0], esz = sdf->dtype == RT_GRID_F16 ? 2 : 4;
     const void* grid = static_cast<const char*>(sdf->grid) + first * n * n * n * esz;
     void* cells = static_cast<char*>(sdf->cells) + first * rtdev::cell_count((int)n, (int)n, (int)n) * 4 * esz;
-    return launch_copies(grid, sdf->dtype, sdf->n, count, cells, nullptr, s);
+    return launch_copies(grid, sdf->dtype, sdf->n, count, 0, cells, nullptr, s);
 }
 
 rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s)
 {
     const int64_t esz = sdf->dtype == RT_GRID_F16 ? 2 : 4;
     const int levels = sdf->levels > 0 ? sdf->levels : 1;
-    rt_status st = own_copy(sdf->cells, sdf->cells_bytes,
-                            levels * rtdev::cell_count(sdf->n[0], sdf->n[1], sdf->n[2]) * 4 * esz);
+    const int64_t entries = rtdev::cell_count(sdf->n[0], sdf->n[1], sdf->n[2]);
+    const int shift = sdf->levels > 0 ? 0 : rtdev::cell_shift(entries, sdf->dtype == RT_GRID_F16);
+    rt_status st = own_copy(sdf->cells, sdf->cells_bytes, levels * (entries << shift) * 4 * esz);
     if (st != RT_OK) return st;
     if (sdf->levels > 0) return rt_launch_cascade_cells(sdf, 0, sdf->levels, s);
     st = own_copy(sdf->pairs, sdf->pairs_bytes, (int64_t)(sdf->n[0] - 1) * sdf->n[1] * sdf->n[2] * 2 * esz);
     if (st != RT_OK) return st;
-    return launch_copies(sdf->grid, sdf->dtype, sdf->n, 1, sdf->cells, sdf->pairs, s);
+    return launch_copies(sdf->grid, sdf->dtype, sdf->n, 1, shift, sdf->cells, sdf->pairs, s);
 }
 
 // Samples up to which a brick is one sample, and up to which it is eight.

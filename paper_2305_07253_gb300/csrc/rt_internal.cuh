@@ -25,7 +25,8 @@
 //   cells  : optional library copy of the grid with the four values of every cell
 //            face across x stored together (16 B float32 / 8 B float16 per entry,
 //            x fastest), so one march step is two adjacent vector loads instead
-//            of eight scalar ones; identical values, identical arithmetic
+//            of eight scalar ones; a large float32 grid's copy holds both faces of
+//            every cell (32 B); identical values, identical arithmetic
 //   pairs  : optional library copy with the two x-neighbours (i, i+1) of every
 //            sample stored together (8 B float32 / 4 B float16, (n0-1) x n1 x n2,
 //            x fastest): a march step is four small loads from a copy twice the
@@ -140,6 +141,8 @@ struct TraceArgs {
     float m_near, m_far;
     int32_t levels;        // 0: one grid; > 0: a cascade read through its cell copy
     int64_t level_cells;   // entries of the cell copy per cascade level
+    int64_t cell_row;      // one grid: bytes from a row of the cell copy to the next,
+    int32_t cell_step;     // and from a cell to its neighbour in x
     CascLevel lv[RT_MAX_LEVELS];
     const float4* rays;
     rt_hit* hits;

@@ -509,13 +509,27 @@ __host__ __device__ __forceinline__ int64_t cell_count(int nx, int ny, int nz)
     return (int64_t)nx * (ny - 1) * (nz - 1);
 }
 
-// the 8 corner values of the cell at entry idx of the copy, order
+// 1: the copy of one grid holds both faces of every cell, entry e (its left face) at
+// 2e and its right one at 2e+1, so that a cell never spans two 32-byte sectors; 0: a
+// face only once.  Once the copy is many times the L2, most loads miss it either way
+// and a float32 cell at an odd entry costs two sectors.  ms per 2,073,600 GI rays,
+// once | both, field only: 320^3 0.513 | 0.604, 384^3 0.671 | 0.705, 448^3 0.866 |
+// 0.773, 512^3 0.985 | 0.824; combined, m = 2: 384^3 0.691 | 0.759, 448^3 0.803 |
+// 0.818, 512^3 0.941 | 0.867.  The line lies at 406^3.  A float16 cell (16 bytes)
+// spans two sectors a quarter of the time: once is faster at 512^3 too (0.695
+// against 0.791 with one 16-byte load per cell).
+__host__ __device__ __forceinline__ int cell_shift(int64_t entries, bool f16)
+{
+    return !f16 && entries >= (1LL << 26) ? 1 : 0;
+}
+
+// the 8 corner values of the cell at this address of the copy, order
 // v000 v100 v010 v110 v001 v101 v011 v111
 template <bool F16>
-__device__ __forceinline__ void load_cell(const void* cells, int64_t idx, float v[8])
+__device__ __forceinline__ void load_cell(const char* cell, float v[8])
 {
     if (F16) {
-        const uint2* q = reinterpret_cast<const uint2*>(cells) + idx;
+        const uint2* q = reinterpret_cast<const uint2*>(cell);
         const uint2 e[2] = {__ldg(q), __ldg(q + 1)};
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
@@ -526,7 +540,7 @@ __device__ __forceinline__ void load_cell(const void* cells, int64_t idx, float 
             v[6 + x] = __high2float(hi);
         }
     } else {
-        const float4* q = reinterpret_cast<const float4*>(cells) + idx;
+        const float4* q = reinterpret_cast<const float4*>(cell);
         const float4 e[2] = {__ldg(q), __ldg(q + 1)};
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
@@ -538,9 +552,10 @@ __device__ __forceinline__ void load_cell(const void* cells, int64_t idx, float 
     }
 }
 
-__device__ __forceinline__ int64_t cell_index(const TraceArgs& a, const Cell& c)
+__device__ __forceinline__ const char* cell_address(const TraceArgs& a, const Cell& c)
 {
-    return cell_slot(c.i0[0], c.i0[1], c.i0[2], a.gn[0], a.gn[1]);
+    return reinterpret_cast<const char*>(a.cells) + a.cell_row * (c.i0[1] + (int64_t)(a.gn[1] - 1) * c.i0[2]) +
+           (int64_t)a.cell_step * c.i0[0];
 }
 
 // the 8 corner values of the cell, order v000 v100 v010 v110 v001 v101 v011 v111
@@ -548,7 +563,7 @@ template <int L>
 __device__ __forceinline__ void corners(const TraceArgs& a, const Cell& c, float v[8])
 {
     if (L == GL_CELLS_F16 || L == GL_CELLS_F32) {
-        load_cell<L == GL_CELLS_F16>(a.cells, cell_index(a, c), v);
+        load_cell<L == GL_CELLS_F16>(cell_address(a, c), v);
         return;
     }
     if (L == GL_PAIRS_F32 || L == GL_PAIRS_F16) {
@@ -673,7 +688,7 @@ __device__ __forceinline__ float casc_trilinear(const TraceArgs& a, int k, float
     float f[3];
     const int64_t idx = casc_locate(a, k, px, py, pz, f);
     float v[8];
-    load_cell<L == GL_CASC_F16>(a.cells, idx, v);
+    load_cell<L == GL_CASC_F16>(reinterpret_cast<const char*>(a.cells) + idx * (L == GL_CASC_F16 ? 8 : 16), v);
     return interp8(f, v);
 }
 
