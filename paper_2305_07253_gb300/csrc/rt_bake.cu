@@ -522,18 +522,6 @@ rt_status launch_copies(const void* grid, int32_t dtype, const int32_t n[3], int
     return RT_OK;
 }
 
-// (re)allocate a library-owned copy
-rt_status own_copy(void*& p, int64_t& have, int64_t bytes)
-{
-    if (p && have == bytes) return RT_OK;
-    if (p) cudaFree(p);
-    p = nullptr;
-    have = 0;
-    RT_CUDA_TRY(cudaMalloc(&p, (size_t)bytes));
-    have = bytes;
-    return RT_OK;
-}
-
 }  // namespace
 
 // cell copies of levels first .. first + count - 1 of a cascade
@@ -545,18 +533,29 @@ rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int first, int count, cudaS
     return launch_copies(grid, sdf->dtype, sdf->n, count, 0, cells, nullptr, s);
 }
 
+// A handle's copies become visible to its traces together, and only once the
+// launch that fills them is enqueued: a handle whose prepare failed is as before it.
 rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s)
 {
     const int64_t esz = sdf->dtype == RT_GRID_F16 ? 2 : 4;
     const int levels = sdf->levels > 0 ? sdf->levels : 1;
     const int64_t entries = rtdev::cell_count(sdf->n[0], sdf->n[1], sdf->n[2]);
     const int shift = sdf->levels > 0 ? 0 : rtdev::cell_shift(entries, sdf->dtype == RT_GRID_F16);
-    rt_status st = own_copy(sdf->cells, sdf->cells_bytes, levels * (entries << shift) * 4 * esz);
-    if (st != RT_OK) return st;
-    if (sdf->levels > 0) return rt_launch_cascade_cells(sdf, 0, sdf->levels, s);
-    st = own_copy(sdf->pairs, sdf->pairs_bytes, (int64_t)(sdf->n[0] - 1) * sdf->n[1] * sdf->n[2] * 2 * esz);
-    if (st != RT_OK) return st;
-    return launch_copies(sdf->grid, sdf->dtype, sdf->n, 1, shift, sdf->cells, sdf->pairs, s);
+    const size_t pairs_bytes = sdf->levels > 0 ? 0 : (size_t)(sdf->n[0] - 1) * sdf->n[1] * sdf->n[2] * 2 * esz;
+    void *cells = sdf->cells, *pairs = sdf->pairs;
+    cudaError_t e = cudaSuccess;
+    if (!cells) e = cudaMalloc(&cells, (size_t)levels * (size_t)(entries << shift) * 4 * esz);
+    if (e == cudaSuccess && !pairs && pairs_bytes) e = cudaMalloc(&pairs, pairs_bytes);
+    rt_status st = e == cudaSuccess ? launch_copies(sdf->grid, sdf->dtype, sdf->n, levels, shift, cells, pairs, s)
+                                    : rt_cuda_fail(e, "allocating the copies of the grid");
+    if (st != RT_OK) {
+        if (cells && !sdf->cells) cudaFree(cells);
+        if (pairs && !sdf->pairs) cudaFree(pairs);
+        return st;
+    }
+    sdf->cells = cells;
+    sdf->pairs = pairs;
+    return RT_OK;
 }
 
 // Samples up to which a brick is one sample, and up to which it is eight.

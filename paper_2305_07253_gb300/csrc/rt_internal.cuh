@@ -78,9 +78,7 @@ struct rt_sdf {
     float lo[3], hi[3], h[3], ih[3];  // one grid; on a cascade: the coarsest level's box
     int32_t n[3];
     void* cells;        // library-owned cell copy (null until rt_sdf_prepare)
-    int64_t cells_bytes;
     void* pairs;        // library-owned x-pair copy (null until rt_sdf_prepare)
-    int64_t pairs_bytes;
     int device;
     // cascade (levels > 0): level k holds n^3 samples at (ilo[k] + i) * h0 * 2^k,
     // stored at grid + k * n^3, its cells at cells + k * n (n-1)^2 entries
