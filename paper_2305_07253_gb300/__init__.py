@@ -37,7 +37,7 @@ LAYOUT_CELLS, LAYOUT_PLAIN, LAYOUT_PAIRS = 0, 1, 2
 EXPORTS = ("rt_scene_build", "rt_scene_info_get", "rt_scene_destroy", "rt_sdf_create", "rt_sdf_destroy",
            "rt_sdf_prepare", "rt_sdf_bake", "rt_trace_bvh", "rt_trace_sdf", "rt_trace_combined",
            "rt_trace_combined_counted", "rt_trace_combined_timed", "rt_trace_combined_noalloc",
-           "rt_trace_combined_backward", "rt_trace_batches", "rt_set_tuning", "rt_get_tuning",
+           "rt_trace_combined_backward", "rt_trace_combined_backward_at", "rt_sdf_version", "rt_trace_batches", "rt_set_tuning", "rt_get_tuning",
            "rt_cascade_create", "rt_cascade_recenter", "rt_cascade_level", "rt_sdf_sites", "rt_trace_combined_host", "rt_scene_export", "rt_last_error",
            "rt_version")
 
@@ -111,6 +111,8 @@ def lib() -> ctypes.CDLL:
             "rt_trace_combined_noalloc": [P, P, P, i64, P, P, P],
             "rt_trace_batches": [P, P, P, i32, P],
             "rt_trace_combined_backward": [P, P, P, i64, P, P, P, P, P],
+            "rt_trace_combined_backward_at": [P, P, ctypes.c_uint64, P, i64, P, P, P, P, P],
+            "rt_sdf_version": [P, P],
             "rt_cascade_create": [P, i32, i32, i32, ctypes.c_float, P, P],
             "rt_cascade_recenter": [P, P, P, P, P],
             "rt_cascade_level": [P, i32, P, P],
@@ -414,14 +416,23 @@ def rt_trace_combined_timed(scene: Scene | None, sdf: Sdf | None, rays: torch.Te
     return hits, [(STAGE_NAMES[kinds[k]], float(ms[k])) for k in range(n.value)]
 
 
+def rt_sdf_version(sdf: Sdf) -> int:
+    """Number of the copies of the grid that traces read (0: none, or not known)."""
+    v = ctypes.c_uint64()
+    _check(lib().rt_sdf_version(sdf.handle, ctypes.byref(v)))
+    return v.value
+
+
 def rt_trace_combined_backward(scene: Scene | None, sdf: Sdf, rays: torch.Tensor, params: rt_split_params,
                                hits: torch.Tensor, grad_t: torch.Tensor, grad_grid: torch.Tensor,
-                               stream=None) -> torch.Tensor:
-    """Adds grad_t * dt/dgrid into grad_grid (float32, grid shape) and returns it."""
+                               stream=None, version: int = 0) -> torch.Tensor:
+    """Adds grad_t * dt/dgrid into grad_grid (float32, grid shape) and returns it.
+    version: rt_sdf_version when the forward call (refine_root, the same rays and
+    params) made the records; while it stands their t are taken as the roots."""
     assert grad_t.dtype == torch.float32 and grad_grid.dtype == torch.float32
-    _check(lib().rt_trace_combined_backward(scene.handle if scene else None, sdf.handle, _dptr(rays), rays.shape[0],
-                                            ctypes.byref(params), _dptr(hits), _dptr(grad_t), _dptr(grad_grid),
-                                            _stream(stream)))
+    _check(lib().rt_trace_combined_backward_at(scene.handle if scene else None, sdf.handle, version, _dptr(rays),
+                                               rays.shape[0], ctypes.byref(params), _dptr(hits), _dptr(grad_t),
+                                               _dptr(grad_grid), _stream(stream)))
     return grad_grid
 
 
@@ -473,6 +484,7 @@ class SdfHitDistance(torch.autograd.Function):
         t = hit_fields(hits)["t"].clone()
         ctx.save_for_backward(rays, hits)
         ctx.scene, ctx.sdf, ctx.params = scene, sdf, p
+        ctx.version = rt_sdf_version(sdf)
         ctx.mark_non_differentiable(hits)
         return t, hits
 
@@ -483,7 +495,7 @@ class SdfHitDistance(torch.autograd.Function):
         if grad_t is None:
             return g, None, None, None, None
         gt = torch.nan_to_num(grad_t.contiguous().float(), nan=0.0, posinf=0.0, neginf=0.0)
-        rt_trace_combined_backward(ctx.scene, ctx.sdf, rays, ctx.params, hits, gt, g)
+        rt_trace_combined_backward(ctx.scene, ctx.sdf, rays, ctx.params, hits, gt, g, version=ctx.version)
         return g, None, None, None, None
 
 

@@ -419,7 +419,7 @@ extern "C" rt_status rt_cascade_recenter(const rt_scene* sc, rt_sdf* sdf, const 
         sdf->hi[a] = hi[a];
     }
     if (moved) *moved = count;
-    return RT_OK;
+    return count > 0 ? rt_copies_written(sdf, s) : RT_OK;
 }
 
 extern "C" rt_status rt_sdf_prepare(rt_sdf* sdf, void* stream)
@@ -667,9 +667,24 @@ extern "C" rt_status rt_trace_combined_counted(const rt_scene* sc, const rt_sdf*
     return trace_common(sc, sdf, rays, n, params, hits, counters, stream);
 }
 
+extern "C" rt_status rt_sdf_version(const rt_sdf* sdf, uint64_t* version)
+{
+    if (!sdf || !version) return rt_fail(RT_ERR_INVALID_ARG, "null argument");
+    *version = sdf->replayed ? 0 : sdf->version;
+    return RT_OK;
+}
+
 extern "C" rt_status rt_trace_combined_backward(const rt_scene* sc, const rt_sdf* sdf, const rt_ray* rays, int64_t n,
                                                 const rt_split_params* params, const rt_hit* hits,
                                                 const float* grad_t, float* grad_grid, void* stream)
+{
+    return rt_trace_combined_backward_at(sc, sdf, 0, rays, n, params, hits, grad_t, grad_grid, stream);
+}
+
+extern "C" rt_status rt_trace_combined_backward_at(const rt_scene* sc, const rt_sdf* sdf, uint64_t version,
+                                                   const rt_ray* rays, int64_t n, const rt_split_params* params,
+                                                   const rt_hit* hits, const float* grad_t, float* grad_grid,
+                                                   void* stream)
 {
     rt_status st = check_params(params);
     if (st != RT_OK) return st;
@@ -688,5 +703,13 @@ extern "C" rt_status rt_trace_combined_backward(const rt_scene* sc, const rt_sdf
     a.rays = reinterpret_cast<const float4*>(rays);
     a.hits = const_cast<rt_hit*>(hits);
     a.n = n;
-    return rt_launch_backward(a, grad_t, grad_grid, (cudaStream_t)stream);
+    // The records' roots stand while the copy they were found in does.  A launch that
+    // a graph replays may meet another copy, and marches.
+    bool at_record = version != 0 && version == sdf->version && !sdf->replayed && a.cells;
+    if (at_record) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        RT_CUDA_TRY(cudaStreamIsCapturing((cudaStream_t)stream, &capture));
+        at_record = capture == cudaStreamCaptureStatusNone;
+    }
+    return rt_launch_backward(a, at_record, grad_t, grad_grid, (cudaStream_t)stream);
 }

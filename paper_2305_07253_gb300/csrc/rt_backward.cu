@@ -3,12 +3,13 @@
 // At a field hit the root p* = o + t d of phi = eps_hit satisfies
 // phi_theta(p*) = eps_hit.  phi is linear in the grid values theta
 // (phi = sum_k w_k(p) theta_k with the trilinear weights w_k), so implicit
-// differentiation gives dt/dtheta_k = -w_k(p*) / (grad phi(p*) . d).  The root is
-// the record's t (a forward call with refine_root); a record whose t is not one
-// (phi does not cross eps_hit there: a forward call without refine_root, or
-// another grid since) is marched again with the forward code (same roundings,
-// same steps) and its root refined in the last step.  grad_t * dt/dtheta_k is
-// scattered into the gradient grid.
+// differentiation gives dt/dtheta_k = -w_k(p*) / (grad phi(p*) . d).  Each ray is
+// marched again with the forward code (same roundings, same steps) and its root
+// refined in the last step, unless the caller's records are of this very copy of
+// the grid (at_record): then the root is the record's t, where phi crosses eps_hit
+// there.  (A crossing alone does not show that it is the first one: the grid may
+// have changed between the two calls.)  grad_t * dt/dtheta_k is scattered into the
+// gradient grid.
 // 1,048,576 rays, 128^3 grid: 249 us with every ray marched again, 54 with the
 // record's root.
 #include "rt_trace_dev.cuh"
@@ -20,8 +21,8 @@ namespace {
 constexpr int kBwdBlock = 128;
 
 template <int L>
-__global__ void __launch_bounds__(kBwdBlock) k_backward(const TraceArgs a, const float* __restrict__ grad_t,
-                                                        float* __restrict__ grad_grid)
+__global__ void __launch_bounds__(kBwdBlock) k_backward(const TraceArgs a, const bool at_record,
+                                                        const float* __restrict__ grad_t, float* __restrict__ grad_grid)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(kBwdBlock) k_backward(const TraceArgs a, const
         return phi < e0;
     };
     bool root = false;
-    if (a.refine_root) root = below(t) ? !below(nextafterf(t, -INFINITY)) : below(nextafterf(t, INFINITY));
+    if (at_record && a.refine_root) root = below(t) ? !below(nextafterf(t, -INFINITY)) : below(nextafterf(t, INFINITY));
     if (root) {
         // a hit at the first sample has no bracket, and its t is the march's start
         float ta = ts, tb = te;
@@ -91,15 +92,15 @@ __global__ void __launch_bounds__(kBwdBlock) k_backward(const TraceArgs a, const
 
 }  // namespace
 
-rt_status rt_launch_backward(const TraceArgs& a, const float* grad_t, float* grad_grid, cudaStream_t s)
+rt_status rt_launch_backward(const TraceArgs& a, bool at_record, const float* grad_t, float* grad_grid, cudaStream_t s)
 {
     const int64_t blocks = (a.n + kBwdBlock - 1) / kBwdBlock;
     if (blocks > 0x7fffffffLL) return rt_fail(RT_ERR_INVALID_ARG, "too many rays");
     // float32 grids only (checked by the caller); the march reads the cell copy when present
     TraceArgs b = a;
     b.pairs = nullptr;
-    if (b.cells) k_backward<GL_CELLS_F32><<<(unsigned)blocks, kBwdBlock, 0, s>>>(b, grad_t, grad_grid);
-    else k_backward<GL_PLAIN_F32><<<(unsigned)blocks, kBwdBlock, 0, s>>>(b, grad_t, grad_grid);
+    if (b.cells) k_backward<GL_CELLS_F32><<<(unsigned)blocks, kBwdBlock, 0, s>>>(b, at_record, grad_t, grad_grid);
+    else k_backward<GL_PLAIN_F32><<<(unsigned)blocks, kBwdBlock, 0, s>>>(b, at_record, grad_t, grad_grid);
     RT_CUDA_TRY(cudaGetLastError());
     return RT_OK;
 }

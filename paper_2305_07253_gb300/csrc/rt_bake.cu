@@ -533,6 +533,16 @@ rt_status rt_launch_cascade_cells(const rt_sdf* sdf, int first, int count, cudaS
     return launch_copies(grid, sdf->dtype, sdf->n, count, 0, cells, nullptr, s);
 }
 
+// A call has written the handle's copies
+rt_status rt_copies_written(rt_sdf* sdf, cudaStream_t s)
+{
+    ++sdf->version;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    RT_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
+    if (capture != cudaStreamCaptureStatusNone) sdf->replayed = true;
+    return RT_OK;
+}
+
 // A handle's copies become visible to its traces together, and only once the
 // launch that fills them is enqueued: a handle whose prepare failed is as before it.
 rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s)
@@ -555,7 +565,7 @@ rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s)
     }
     sdf->cells = cells;
     sdf->pairs = pairs;
-    return RT_OK;
+    return rt_copies_written(sdf, s);
 }
 
 // Samples up to which a brick is one sample, and up to which it is eight.

@@ -79,6 +79,8 @@ struct rt_sdf {
     int32_t n[3];
     void* cells;        // library-owned cell copy (null until rt_sdf_prepare)
     void* pairs;        // library-owned x-pair copy (null until rt_sdf_prepare)
+    uint64_t version;   // how often the copies have been written (rt_sdf_version)
+    bool replayed;      // a graph may write them again without this handle knowing
     int device;
     // cascade (levels > 0): level k holds n^3 samples at (ilo[k] + i) * h0 * 2^k,
     // stored at grid + k * n^3, its cells at cells + k * n (n-1)^2 entries
@@ -259,7 +261,8 @@ constexpr int kSmallBlock = 128;                // their threads per block, what
 // conc_set: the set of library streams a concurrent program of this call uses
 rt_status rt_launch_trace(const TraceArgs& a, bool counted, cudaStream_t s, StageTiming* timing = nullptr,
                           int conc_set = 0);
-rt_status rt_launch_backward(const TraceArgs& a, const float* grad_t, float* grad_grid, cudaStream_t s);
+// at_record: the records' t are the roots of the copy that the march reads
+rt_status rt_launch_backward(const TraceArgs& a, bool at_record, const float* grad_t, float* grad_grid, cudaStream_t s);
 rt_status rt_build_scene(const float* verts, int64_t nv, const int32_t* tris, int64_t nt, cudaStream_t s,
                          rt_scene* out);
 rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, cudaStream_t s);
@@ -312,6 +315,7 @@ rt_status rt_build_wide(rt_scene* sc, const int2* child, const int2* range, cons
                         const float4* node_hi, const float4* leaf_lo, const float4* leaf_hi, float pad,
                         const WideScratch& ws, cudaStream_t s);
 rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s);
+rt_status rt_copies_written(rt_sdf* sdf, cudaStream_t s);
 rt_status rt_treelet_optimise(int64_t nt, int passes, int2* child, int2* range, int32_t* par_i, int32_t* par_l,
                               int32_t* order, float4* llo, float4* lhi, float4* nlo, float4* nhi, float* cost,
                               const TreeletScratch& ws, cudaStream_t s);
