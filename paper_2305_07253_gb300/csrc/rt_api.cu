@@ -322,6 +322,7 @@ extern "C" rt_status rt_cascade_create(const void* d_grid, int32_t dtype, int32_
     g->dtype = dtype;
     g->levels = levels;
     g->h0 = h0;
+    g->bake_method = RT_BAKE_BVH;  // of new samples beside values that the caller wrote
     for (int k = 0; k < levels; ++k) {
         if (!cascade_origin(center, h0, n, k, g->ilo[k])) {
             delete g;

@@ -723,14 +723,14 @@ static rt_status launch_brute(const BakeArgs& b, cudaStream_t s)
 // search 0.7 to 1.5 ns (123,000 samples: 344 triangles 0.12 and 0.10 ms, 11,748
 // triangles 4.1 and 0.18 ms), and the search gives the same values.
 constexpr int64_t kBruteMost = 256;
+static bool brute_values(const BakeArgs& b, int32_t method)
+{
+    return method == RT_BAKE_BRUTE || (method == RT_BAKE_AUTO && (double)b.count * (double)b.n_tris <= 17179869184.0);
+}
 static bool pick_brute(BakeArgs& b, int32_t method)
 {
-    if (method == RT_BAKE_AUTO) {
-        if ((double)b.count * (double)b.n_tris > 17179869184.0) return false;
-        b.brute_sum = 1;
-        return b.n_tris <= kBruteMost;
-    }
-    return method == RT_BAKE_BRUTE;
+    b.brute_sum = brute_values(b, method);
+    return method == RT_BAKE_BRUTE || (b.brute_sum && b.n_tris <= kBruteMost);
 }
 
 static BakeArgs bake_args(const rt_scene* sc, const rt_sdf* sdf)
@@ -773,11 +773,13 @@ static void coarser_source(BakeArgs& b, const rt_sdf* sdf, int k)
 
 // Bake of cascade level k of a moved cascade: the kept samples from `keep` and
 // the new slabs (keep non-null), or the whole level, bounded by the values of
-// the next coarser level.
+// the next coarser level.  New samples get the values that the method of the
+// cascade's last bake gives them, so that a rolled level equals a fresh one.
 rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, const void* keep, const int32_t shift[3],
                                  cudaStream_t s)
 {
     BakeArgs b = level_args(sc, sdf, k);
+    b.brute_sum = brute_values(b, sdf->bake_method);
     const int32_t n = sdf->n[0];
     if (keep) {
         const unsigned threads = n >= 128 ? 128 : (n >= 64 ? 64 : 32);
