@@ -43,6 +43,10 @@ __device__ __forceinline__ float dot3r(const float* a, const float* b)
 // mostly fall in different regions, so there are no branches: the region picks
 // the operands of one division and of q = (base + s1 dir1) + s2 dir2.  A vertex
 // has s1 = s2 = 0 and an edge s2 = 0, which leave base + s1 dir1 as it is.
+// Infinite where it is not a number: a triangle with two equal vertices divides by
+// the length of their edge at half of all positions.  A distance that compares with
+// every other is what makes the best site independent of the order in which the
+// steps meet the candidates.
 __device__ __forceinline__ float tri_d2_rn(const float* p, const float* a, const float* b, const float* c)
 {
     float ab[3], ac[3], ap[3], bp[3], cp[3];
@@ -85,7 +89,7 @@ __device__ __forceinline__ float tri_d2_rn(const float* p, const float* a, const
         const float q = __fadd_rn(__fadd_rn(base, __fmul_rn(s1, dir)), __fmul_rn(s2, ac[k]));
         pq[k] = __fsub_rn(p[k], q);
     }
-    return dot3r(pq, pq);
+    return fminf(dot3r(pq, pq), __int_as_float(0x7f800000));  // (the minimum of a NaN and a number is the number)
 }
 
 // Separation along an axis on which the triangle's vertices lie at p0, p1, p2 and
