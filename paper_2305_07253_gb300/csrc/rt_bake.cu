@@ -9,7 +9,8 @@
 //
 // Two methods with the same result: brute force (every triangle, staged through
 // shared memory in tiles) and a BVH-pruned nearest query, which a warp runs for
-// up to 32 neighbouring samples together (k_bake_bricks).
+// up to 32 neighbouring samples together (k_bake_bricks), or, with few triangles,
+// a thread for one sample (k_bake_threads).
 #include <math.h>
 #include <string.h>
 
@@ -223,8 +224,7 @@ __device__ __forceinline__ void brick_pairs(const BakeArgs& b, BrickShared& w, i
         const float3 p = xyz(ps);
         float3 q;
         closest_point_rn(p, xyz(a), xyz(w.v1[i]), xyz(w.v2[i]), q);
-        const float3 pq = sub(p, q);
-        const float d2 = b.brute_sum ? __fmaf_rn(pq.z, pq.z, __fmaf_rn(pq.y, pq.y, __fmul_rn(pq.x, pq.x))) : dot_rn(pq, pq);
+        const float d2 = gap2_rn(p, q, b.brute_sum);
         if (d2 <= ps.w) atomicMin(&w.key[s], (unsigned long long)__float_as_uint(d2) << 32 | __float_as_uint(a.w));
     }
     __syncwarp();
@@ -445,6 +445,102 @@ __global__ void __launch_bounds__(32 * kBrickWarps, 16) k_bake_bricks(const Bake
     }
 }
 
+// Few triangles (few_triangles): one traversal per thread, whose path is shorter than
+// the fixed steps of a brick's search.  What bounds it is the latency of the nodes and
+// triangles of the longest path.  A sample searches within the bound that its source's
+// value gives, so no sites are kept and no scratch is needed.
+struct ThreadPass {
+    int32_t sub;        // > 0: only the samples whose indices are multiples of it
+    int32_t own;        // > 0: the source is this grid's own samples at that stride, which are left as they are
+    const void* keep;   // rolling update: sample i takes the value of sample i + shift of it wherever that lies
+    int32_t shift[3];   // inside the level (the level before the move)
+};
+
+// nearest triangle to p among those at most sqrt(d2_start) away; k = -1 when there is none
+__device__ __forceinline__ Nearest nearest_triangle(const BakeArgs& b, float3 p, float d2_start)
+{
+    Nearest nb = {d2_start, -1, 0x7fffffff};
+    int32_t stack[RT_STACK_DEPTH];
+    float reach[RT_STACK_DEPTH];
+    int sp = 0;
+    int32_t node = b.n_tris > 1 ? 0 : ~0;
+    // bounded by the number of nodes; the guard stops only a corrupt structure
+    for (uint32_t guard = 0; guard < (1u << 26); ++guard) {
+        if (node >= 0) {
+            float v[8], u[8];
+            rtdev::load_node(b.nodes, node, v, u);
+            const float d0 = box_d2(v[0], v[1], v[2], v[3], u[0], u[1], p), d1 = box_d2(v[4], v[5], v[6], v[7], u[2], u[3], p);
+            const int32_t c0 = __float_as_int(u[4]), c1 = __float_as_int(u[5]);
+            const bool in0 = d0 <= nb.d2, in1 = d1 <= nb.d2;
+            if (in0 && in1) {
+                if (sp < RT_STACK_DEPTH) {
+                    stack[sp] = d1 < d0 ? c0 : c1;
+                    reach[sp++] = fmaxf(d0, d1);
+                }
+                node = d1 < d0 ? c1 : c0;
+                continue;
+            }
+            if (in0 || in1) {
+                node = in0 ? c0 : c1;
+                continue;
+            }
+        } else {
+            consider_rn(nb, p, b.tris, ~node, b.brute_sum);
+        }
+        bool more = false;
+        while (sp > 0 && !more) {
+            --sp;
+            more = reach[sp] <= nb.d2;
+        }
+        if (!more) break;
+        node = stack[sp];
+    }
+    return nb;
+}
+
+__global__ void __launch_bounds__(kBakeBlock) k_bake_threads(const BakeArgs b, const ThreadPass tp)
+{
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int32_t step = tp.sub > 0 ? tp.sub : 1;
+    const int64_t mx = (b.n[0] - 1) / step + 1, my = (b.n[1] - 1) / step + 1, mz = (b.n[2] - 1) / step + 1;
+    if (t >= mx * my * mz) return;
+    const int32_t ii[3] = {(int32_t)(t % mx) * step, (int32_t)((t / mx) % my) * step, (int32_t)(t / (mx * my)) * step};
+    const int64_t i = sample_index(b, ii);
+    if (tp.keep) {
+        const int32_t x = ii[0] + tp.shift[0], y = ii[1] + tp.shift[1], z = ii[2] + tp.shift[2];
+        if (x >= 0 && x < b.n[0] && y >= 0 && y < b.n[1] && z >= 0 && z < b.n[2]) {
+            const int64_t src = x + (int64_t)b.n[0] * (y + (int64_t)b.n[1] * z);
+            if (b.f16) reinterpret_cast<__half*>(b.grid)[i] = reinterpret_cast<const __half*>(tp.keep)[src];
+            else reinterpret_cast<float*>(b.grid)[i] = reinterpret_cast<const float*>(tp.keep)[src];
+            return;
+        }
+    }
+    float bound;
+    if (tp.own > 0) {
+        // the nearest sample of the first pass, whose values stand in this grid
+        int32_t src[3];
+        float d2 = 0.f;
+        bool self = true;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const int32_t most = (b.n[a] - 1) / tp.own;
+            const int32_t j = min((ii[a] + tp.own / 2) / tp.own, most);
+            src[a] = j * tp.own;
+            const float gap = (float)(ii[a] - src[a]) * b.h[a];
+            d2 += gap * gap;
+            self = self && src[a] == ii[a];
+        }
+        if (self) return;
+        bound = (fabsf(load_value(b.grid, b.f16, sample_index(b, src))) + sqrtf(d2)) * 1.002f + 1e-6f;
+    } else {
+        bound = distance_bound(b, ii);
+    }
+    const float3 p = sample_pos(b, ii);
+    Nearest nb = nearest_triangle(b, p, bound * bound);
+    if (nb.k < 0 && !isinf(bound)) nb = nearest_triangle(b, p, __int_as_float(0x7f800000));  // a bound that held no triangle
+    store(b, i, signed_distance_rn(p, nb, b.tris, b.pn));
+}
+
 // rolling update: sample i takes the value of sample i + shift of `keep` (the
 // level before the move) wherever that lies inside the level
 __global__ void k_roll(const void* keep, void* grid, int32_t f16, int32_t n, int3 shift)
@@ -568,20 +664,29 @@ rt_status rt_launch_prepare(rt_sdf* sdf, cudaStream_t s)
     return rt_copies_written(sdf, s);
 }
 
-// Samples up to which a brick is one sample, and up to which it is eight.
-// Measured, ms: a 5 x 32^3 cascade of the frame scene (32,768 samples a level)
-// 0.90 with one, 1.31 with eight; 41^3 to 64^3 grids 0.42-0.50 with eight, 0.92-1.0
-// with 32; 97^3 samples, 1,213,548 triangles 2.0 with eight, 2.1 with 32; 256^3
-// samples 18.0 with eight, 11.2 with 32.
-constexpr int64_t kSingleMost = 32768;
-constexpr int64_t kEightMost = 524288;
 constexpr int kSubStride = 4;  // first-pass sub-lattice of a bake without a source
 
-// Bricks of 32 samples (4 x 4 x 2) do the least work; bricks of one sample finish
-// soonest.  A launch with few samples lasts as long as its slowest brick (one
-// near the centre of a round object), so the fewer the samples the smaller the
-// bricks.
-static int brick_log2(int64_t samples) { return samples <= kSingleMost ? 0 : (samples <= kEightMost ? 3 : 5); }
+// log2 of a brick's samples.  Bricks of 32 samples (4 x 4 x 2) do the least work;
+// bricks of one sample finish soonest.  A launch with few samples lasts as long as
+// its slowest brick (one near the centre of a round object), so the fewer the
+// samples the smaller the bricks: one sample up to 32,768, eight up to 2^19.  ms: a
+// 5 x 32^3 cascade of the frame scene (32,768 samples a level) 0.90 with one, 1.31
+// with eight; 41^3 to 64^3 grids 0.42-0.50 with eight, 0.92-1.0 with 32; 97^3
+// samples, 1,213,548 triangles 2.0 with eight, 2.1 with 32; 256^3 samples 18.0 with
+// eight, 11.2 with 32.
+// With few triangles no brick is slow, and the number of bricks counts: one sample
+// up to 6,144 and, where the search starts from a value and not from a triangle,
+// eight up to 2^17.  us at 10,300 triangles (eight spheres), the limits above |
+// these: 32^3 113 | 83, 5 x 32^3 401 | 280, moves of 5 x 64^3 by 1 and 40 samples 113
+// | 106 and 476 | 463, of 5 x 128^3 by 10 542 | 395.  At 20,540 triangles moves of 5
+// x 32^3 by 10 and of 5 x 64^3 by 40 were slower with them (250 | 283, 645 | 716).
+constexpr int64_t kFewTriangles = 16384;
+static int brick_log2(const BakeArgs& b, int64_t samples)
+{
+    const bool few = b.n_tris <= kFewTriangles;
+    if (samples <= (few ? 6144 : 32768)) return 0;
+    return samples <= (few && b.bsrc ? 131072 : 524288) ? 3 : 5;
+}
 
 // cut the box into bricks of 2^lg samples, as cubic as the box allows
 static void set_bricks(PacketGrid& pg, PacketBox& bx, int lg)
@@ -607,7 +712,7 @@ static void set_bricks(PacketGrid& pg, PacketBox& bx, int lg)
 }
 
 // whole grid, or every `sub`-th sample of it
-static PacketGrid whole_grid(const int32_t n[3], int sub)
+static PacketGrid whole_grid(const BakeArgs& b, int sub)
 {
     PacketGrid pg;
     memset(&pg, 0, sizeof(pg));
@@ -615,18 +720,19 @@ static PacketGrid whole_grid(const int32_t n[3], int sub)
     pg.sub = sub;
     int64_t samples = 1;
     for (int a = 0; a < 3; ++a) {
-        pg.box[0].dim[a] = (n[a] - 1) / sub + 1;
+        pg.box[0].dim[a] = (b.n[a] - 1) / sub + 1;
         samples *= pg.box[0].dim[a];
     }
-    pg.brick_log2 = brick_log2(samples);
+    pg.brick_log2 = brick_log2(b, samples);
     set_bricks(pg, pg.box[0], pg.brick_log2);
     return pg;
 }
 
 // the samples of an n^3 level that a move by `shift` samples brings in: an x slab,
 // the y slab of the rest, the z slab of that rest
-static PacketGrid new_slabs(int32_t n, const int32_t shift[3])
+static PacketGrid new_slabs(const BakeArgs& b, const int32_t shift[3])
 {
+    const int32_t n = b.n[0];
     PacketGrid pg;
     memset(&pg, 0, sizeof(pg));
     pg.sub = 1;
@@ -644,7 +750,7 @@ static PacketGrid new_slabs(int32_t n, const int32_t shift[3])
         lo[a] = shift[a] > 0 ? 0 : thick;
         dim[a] -= thick;
     }
-    pg.brick_log2 = brick_log2((int64_t)n * n * n - (int64_t)dim[0] * dim[1] * dim[2]);
+    pg.brick_log2 = brick_log2(b, (int64_t)n * n * n - (int64_t)dim[0] * dim[1] * dim[2]);
     for (int k = 0; k < pg.boxes; ++k) set_bricks(pg, pg.box[k], pg.brick_log2);
     return pg;
 }
@@ -662,6 +768,30 @@ static rt_status launch_packets(const BakeArgs& b, const PacketGrid& pg, cudaStr
     }
     RT_CUDA_TRY(cudaGetLastError());
     return RT_OK;
+}
+
+static rt_status launch_threads(const BakeArgs& b, const ThreadPass& tp, cudaStream_t s)
+{
+    int64_t samples = 1;
+    for (int a = 0; a < 3; ++a) samples *= (b.n[a] - 1) / (tp.sub > 0 ? tp.sub : 1) + 1;
+    const int64_t blocks = (samples + kBakeBlock - 1) / kBakeBlock;
+    if (blocks > 0x7fffffffLL) return rt_fail(RT_ERR_INVALID_ARG, "grid too large for one launch");
+    k_bake_threads<<<(unsigned)blocks, kBakeBlock, 0, s>>>(b, tp);
+    RT_CUDA_TRY(cudaGetLastError());
+    return RT_OK;
+}
+
+// the stride-4 sub-lattice first, then every other sample within the bound of its
+// nearest sub-lattice sample
+static rt_status launch_threads_two_pass(const BakeArgs& b, cudaStream_t s)
+{
+    ThreadPass tp = {};
+    tp.sub = kSubStride;
+    const rt_status st = launch_threads(b, tp, s);
+    if (st != RT_OK) return st;
+    tp.sub = 0;
+    tp.own = kSubStride;
+    return launch_threads(b, tp, s);
 }
 
 // device scratch of one bake, returned in stream order
@@ -693,7 +823,7 @@ static rt_status launch_two_pass(BakeArgs b, int32_t* sub_sites, cudaStream_t s)
     b.sdst = sub_sites;
     b.ssrc = nullptr;
     b.bsrc = nullptr;
-    const PacketGrid coarse = whole_grid(b.n, kSubStride);
+    const PacketGrid coarse = whole_grid(b, kSubStride);
     rt_status st = launch_packets(b, coarse, s);
     if (st != RT_OK) return st;
     b.grid = grid;
@@ -705,7 +835,7 @@ static rt_status launch_two_pass(BakeArgs b, int32_t* sub_sites, cudaStream_t s)
         b.bilo[a] = 0;
         b.bdim[a] = coarse.box[0].dim[a];
     }
-    return launch_packets(b, whole_grid(b.n, 1), s);
+    return launch_packets(b, whole_grid(b, 1), s);
 }
 
 static rt_status launch_brute(const BakeArgs& b, cudaStream_t s)
@@ -732,6 +862,15 @@ static bool pick_brute(BakeArgs& b, int32_t method)
     b.brute_sum = brute_values(b, method);
     return method == RT_BAKE_BRUTE || (b.brute_sum && b.n_tris <= kBruteMost);
 }
+
+// Up to 512 triangles, 1,024 on a cascade's levels and over 2^22 samples, a thread
+// searches for a sample.
+// us, threads | bricks, 24 triangles: 256^3 762 | 1,319, 5 x 64^3 141 | 399, its moves
+// by 1 and 40 samples 74 | 87 and 143 | 190; 252 triangles: 256^3 1,441 | 1,734, 5 x
+// 64^3 244 | 456, moves 86 | 96 and 214 | 242; 700 triangles: 32^3 201 | 66, 64^3 160 |
+// 130, 256^3 1,384 | 1,584, 5 x 64^3 293 | 442, moves 87 | 92 and 210 | 247; 1,340
+// triangles: 64^3 253 | 127, 5 x 64^3 556 | 494, moves 107 | 104 and 334 | 286.
+static bool few_triangles(const BakeArgs& b, bool level) { return b.n_tris <= (level || b.count > (1 << 22) ? 1024 : 512); }
 
 static BakeArgs bake_args(const rt_scene* sc, const rt_sdf* sdf)
 {
@@ -771,6 +910,19 @@ static void coarser_source(BakeArgs& b, const rt_sdf* sdf, int k)
     for (int a = 0; a < 3; ++a) b.bilo[a] = sdf->ilo[k + 1][a];
 }
 
+static void coarser_values(BakeArgs& b, const rt_sdf* sdf, int k)
+{
+    b.bsrc = static_cast<const char*>(sdf->grid) + (k + 1) * b.count * (b.f16 ? 2 : 4);
+    coarser_source(b, sdf, k);
+}
+
+static rt_status whole_level_by_threads(BakeArgs b, const rt_sdf* sdf, int k, cudaStream_t s)
+{
+    if (k + 1 >= sdf->levels) return launch_threads_two_pass(b, s);
+    coarser_values(b, sdf, k);
+    return launch_threads(b, ThreadPass{}, s);
+}
+
 // Bake of cascade level k of a moved cascade: the kept samples from `keep` and
 // the new slabs (keep non-null), or the whole level, bounded by the values of
 // the next coarser level.  New samples get the values that the method of the
@@ -781,7 +933,18 @@ rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, c
     BakeArgs b = level_args(sc, sdf, k);
     b.brute_sum = brute_values(b, sdf->bake_method);
     const int32_t n = sdf->n[0];
+    const bool threads = few_triangles(b, true);
     if (keep) {
+        if (threads) {
+            b.bsrc = keep;
+            ThreadPass tp = {};
+            tp.keep = keep;
+            for (int a = 0; a < 3; ++a) {
+                tp.shift[a] = shift[a];
+                b.bilo[a] = sdf->ilo[k][a] - shift[a];
+            }
+            return launch_threads(b, tp, s);
+        }
         const unsigned threads = n >= 128 ? 128 : (n >= 64 ? 64 : 32);
         k_roll<<<dim3((n + threads - 1) / threads, n, n), threads, 0, s>>>(keep, b.grid, b.f16, n,
                                                                            make_int3(shift[0], shift[1], shift[2]));
@@ -789,12 +952,12 @@ rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, c
         // new samples are bounded by the nearest kept sample
         b.bsrc = keep;
         for (int a = 0; a < 3; ++a) b.bilo[a] = sdf->ilo[k][a] - shift[a];
-        return launch_packets(b, new_slabs(n, shift), s);
+        return launch_packets(b, new_slabs(b, shift), s);
     }
+    if (threads) return whole_level_by_threads(b, sdf, k, s);
     if (k + 1 < sdf->levels) {
-        b.bsrc = static_cast<const char*>(sdf->grid) + (k + 1) * b.count * (b.f16 ? 2 : 4);
-        coarser_source(b, sdf, k);
-        return launch_packets(b, whole_grid(b.n, 1), s);
+        coarser_values(b, sdf, k);
+        return launch_packets(b, whole_grid(b, 1), s);
     }
     BakeScratch scratch(s);
     const rt_status st = scratch.take(sub_sites_bytes(b.n));
@@ -813,6 +976,7 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
             b.h[k] = sdf->h[k];
         }
         if (pick_brute(b, method)) return launch_brute(b, s);
+        if (few_triangles(b, false)) return launch_threads_two_pass(b, s);
         rt_status st = scratch.take(sub_sites_bytes(b.n));
         if (st != RT_OK) return st;
         return launch_two_pass(b, static_cast<int32_t*>(scratch.p), s);
@@ -821,6 +985,16 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
     if (pick_brute(first, method)) {
         for (int k = sdf->levels - 1; k >= 0; --k) {
             rt_status st = launch_brute(level_args(sc, sdf, k), s);
+            if (st != RT_OK) return st;
+        }
+        return RT_OK;
+    }
+    if (few_triangles(first, true)) {
+        // coarsest first: each level bounds the next finer one
+        for (int k = sdf->levels - 1; k >= 0; --k) {
+            BakeArgs b = level_args(sc, sdf, k);
+            b.brute_sum = first.brute_sum;
+            const rt_status st = whole_level_by_threads(b, sdf, k, s);
             if (st != RT_OK) return st;
         }
         return RT_OK;
@@ -843,7 +1017,7 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
         } else {
             b.ssrc = sites[(k + 1) & 1];
             coarser_source(b, sdf, k);
-            st = launch_packets(b, whole_grid(b.n, 1), s);
+            st = launch_packets(b, whole_grid(b, 1), s);
         }
         if (st != RT_OK) return st;
     }

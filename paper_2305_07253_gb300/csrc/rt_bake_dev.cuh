@@ -119,13 +119,19 @@ __device__ __forceinline__ void consider(Nearest& nb, float3 p, const float4* tr
     }
 }
 
-__device__ __forceinline__ void consider_rn(Nearest& nb, float3 p, const float4* tris, int32_t k)
+// the squared distance between p and q, in the order of the brute force kernel's sum or in dot_rn's
+__device__ __forceinline__ float gap2_rn(float3 p, float3 q, bool brute_sum)
+{
+    const float3 pq = sub(p, q);
+    return brute_sum ? __fmaf_rn(pq.z, pq.z, __fmaf_rn(pq.y, pq.y, __fmul_rn(pq.x, pq.x))) : dot_rn(pq, pq);
+}
+
+__device__ __forceinline__ void consider_rn(Nearest& nb, float3 p, const float4* tris, int32_t k, bool brute_sum)
 {
     const float4 v0 = __ldg(tris + 3 * (int64_t)k), v1 = __ldg(tris + 3 * (int64_t)k + 1), v2 = __ldg(tris + 3 * (int64_t)k + 2);
     float3 q;
     closest_point_rn(p, xyz(v0), xyz(v1), xyz(v2), q);
-    const float3 pq = sub(p, q);
-    const float d2 = dot_rn(pq, pq);
+    const float d2 = gap2_rn(p, q, brute_sum);
     const int32_t prim = __float_as_int(v0.w);
     if (d2 < nb.d2 || (d2 == nb.d2 && prim < nb.prim)) {
         nb.d2 = d2;
