@@ -329,7 +329,8 @@ __global__ void __launch_bounds__(128) k_refine(const TraceArgs a)
 // ---------------------------------------------------------------------------
 struct DeviceInfo {
     int sms = 0;
-    cudaMemPool_t pool = nullptr;
+    cudaMemPool_t pool = nullptr;     // of the traces
+    cudaMemPool_t scratch = nullptr;  // of builds and bakes (rt_scratch_alloc)
 };
 
 std::mutex g_mu;
@@ -353,6 +354,11 @@ rt_status device_info(DeviceInfo*& out)
         // keep freed scratch in the pool between calls instead of returning it
         uint64_t keep = ~0ull;
         RT_CUDA_TRY(cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        // builds and bakes on many streams at once hold more for a while; what exceeds
+        // this goes back at the next synchronisation
+        RT_CUDA_TRY(cudaMemPoolCreate(&d.scratch, &props));
+        keep = 2 * kScratchKept;
+        RT_CUDA_TRY(cudaMemPoolSetAttribute(d.scratch, cudaMemPoolAttrReleaseThreshold, &keep));
     }
     out = &d;
     return RT_OK;
@@ -685,7 +691,7 @@ rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s)
     DeviceInfo* dev = nullptr;
     const rt_status st = device_info(dev);
     if (st != RT_OK) return st;
-    RT_CUDA_TRY(cudaMallocFromPoolAsync(p, bytes, dev->pool, s));
+    RT_CUDA_TRY(cudaMallocFromPoolAsync(p, bytes, dev->scratch, s));
     return RT_OK;
 }
 
