@@ -381,7 +381,8 @@ rt_status launch_stage(const TraceArgs& a, const StageArgs& st, const rt_tuning&
 {
     const bool field = st.kind == ST_FIELD_FULL || st.kind == ST_FIELD_SPLIT;
     if (field) {
-        switch (grid_layout_of(a)) {
+        const int layout = grid_layout_of(a);
+        switch (layout == GL_CELLS_F32 && a.cell_step == 16 ? GL_ONCE_F32 : layout) {
 #define RT_FIELD_CASE(LL)                                                                  \
     case LL: {                                                                             \
         int blocks = persistent_blocks(k_stage_field<COUNT, LL>, tu.block, tu, sms);       \
@@ -397,6 +398,7 @@ rt_status launch_stage(const TraceArgs& a, const StageArgs& st, const rt_tuning&
             RT_FIELD_CASE(GL_PAIRS_F16)
             RT_FIELD_CASE(GL_CASC_F32)
             RT_FIELD_CASE(GL_CASC_F16)
+            RT_FIELD_CASE(GL_ONCE_F32)
 #undef RT_FIELD_CASE
         }
     } else if (a.wnodes) {

@@ -440,9 +440,12 @@ __device__ __forceinline__ bool bvh_segment(const TraceArgs& a, float3 o, float3
 // ---------------------------------------------------------------------------
 // Grid storage seen by the march, fixed at compile time so that a step has no
 // layout or type branches: the caller's plain grid (float32 / float16) or the
-// library's cell copy (float32 / float16).
+// library's cell copy (float32 / float16).  GL_ONCE_F32 is the float32 copy whose
+// faces stand once, with that step known: the field stage takes it (2,073,600 GI rays,
+// field only, grid 64^3 336 us with the step read from the arguments, 329 with it
+// known; 128^3 345, 339; one thread per query is no faster with it).
 enum GridLayout { GL_PLAIN_F32 = 0, GL_PLAIN_F16 = 1, GL_CELLS_F32 = 2, GL_CELLS_F16 = 3, GL_PAIRS_F32 = 4,
-                  GL_PAIRS_F16 = 5, GL_CASC_F32 = 6, GL_CASC_F16 = 7 };
+                  GL_PAIRS_F16 = 5, GL_CASC_F32 = 6, GL_CASC_F16 = 7, GL_ONCE_F32 = 8 };
 
 __host__ __device__ constexpr bool is_cascade(int L) { return L == GL_CASC_F32 || L == GL_CASC_F16; }
 
@@ -552,18 +555,19 @@ __device__ __forceinline__ void load_cell(const char* cell, float v[8])
     }
 }
 
+template <int L>
 __device__ __forceinline__ const char* cell_address(const TraceArgs& a, const Cell& c)
 {
     return reinterpret_cast<const char*>(a.cells) + a.cell_row * (c.i0[1] + (int64_t)(a.gn[1] - 1) * c.i0[2]) +
-           (int64_t)a.cell_step * c.i0[0];
+           (int64_t)(L == GL_ONCE_F32 ? 16 : a.cell_step) * c.i0[0];
 }
 
 // the 8 corner values of the cell, order v000 v100 v010 v110 v001 v101 v011 v111
 template <int L>
 __device__ __forceinline__ void corners(const TraceArgs& a, const Cell& c, float v[8])
 {
-    if (L == GL_CELLS_F16 || L == GL_CELLS_F32) {
-        load_cell<L == GL_CELLS_F16>(cell_address(a, c), v);
+    if (L == GL_CELLS_F16 || L == GL_CELLS_F32 || L == GL_ONCE_F32) {
+        load_cell<L == GL_CELLS_F16>(cell_address<L>(a, c), v);
         return;
     }
     if (L == GL_PAIRS_F32 || L == GL_PAIRS_F16) {
