@@ -524,7 +524,8 @@ rt_status run_concurrent(const TraceArgs& a, const int kinds[3], int n_st, const
     rt_tuning tn = tu, tf = tu;
     if (tu.blocks_per_sm == 0) {
         tn.blocks_per_sm = a.levels > 0 ? kConcNearCascade : kConcNearBlocks;
-        tf.blocks_per_sm = a.levels > 0 ? kConcFieldCascade : kConcFieldBlocks;
+        const bool both = a.cells && !a.grid_f16 && a.cell_step == 32;
+        tf.blocks_per_sm = a.levels > 0 ? kConcFieldCascade : (both ? kConcFieldBoth : kConcFieldBlocks);
     }
     // near stream: the order, then the near stage
     TraceArgs ao = a;
