@@ -402,10 +402,10 @@ enum { RT_MAX_BATCHES = 16 };
  *   - at most RT_MAX_BATCHES batches, at most 2^31-1 queries in total;
  *   - mode, any_hit, m_near and m_far may differ per batch; max_steps,
  *     hit_eps_vox, min_step_vox and refine_root must be equal in all batches;
- *   - with at most 131,072 queries in all, one launch of one thread per query
- *     serves the call, unless the tuning's kernel is RT_KERNEL_WAVEFRONT;
- *     otherwise the wavefront stage kernels do; the tuning's block, residency,
- *     refill and layout apply.
+ *   - with at most 524,288 queries in all (131,072 if no batch reads the grid),
+ *     one launch of one thread per query serves the call, unless the tuning's
+ *     kernel is RT_KERNEL_WAVEFRONT; otherwise the wavefront stage kernels do;
+ *     the tuning's block, residency, refill and layout apply.
  * Errors: RT_ERR_INVALID_ARG before any work for bad batches. */
 rt_status rt_trace_batches(const rt_scene* scene, const rt_sdf* sdf, const rt_batch* batches, int32_t n_batches,
                            void* stream);

@@ -463,9 +463,8 @@ extern "C" rt_status rt_trace_batches(const rt_scene* sc, const rt_sdf* sdf, con
     rt_apply_layout(a, tu);
     a.n = total;
     a.counters = nullptr;
-    if (tu.kernel != RT_KERNEL_WAVEFRONT && total <= kSmallCall) {
-        // every query resident at once: the pipeline's launches would cost more
-        // than regrouping gains (rt_launch_trace)
+    if (tu.kernel != RT_KERNEL_WAVEFRONT && total <= (need_grid ? kSmallBatch : kSmallCall)) {
+        // the pipeline's launches would cost more than regrouping gains
         if (a.wnodes) launch_batch_simple<true>(a, tb, kSmallBlock, (cudaStream_t)stream);
         else launch_batch_simple<false>(a, tb, kSmallBlock, (cudaStream_t)stream);
         RT_CUDA_TRY(cudaGetLastError());

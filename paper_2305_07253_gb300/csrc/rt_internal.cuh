@@ -259,6 +259,11 @@ rt_status rt_scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 // resident at once (rt_launch_trace has the figures)
 constexpr int64_t kSmallCall = 131072;
 constexpr int64_t kSmallCallTriangles = 65536;  // calls that trace triangles only
+// For batches, whose pipeline has more launches (those that trace triangles only:
+// kSmallCall).  us, pipeline | one thread per query, frame scene, 256^3, at 150,000,
+// 260,000 and 520,000 queries: GI 201 | 150, 240 | 218, 280 | 282; GI and shadow 257 |
+// 155, 283 | 190, 328 | 274; the four kinds of a frame 213 | 147, 250 | 190, 272 | 207.
+constexpr int64_t kSmallBatch = 524288;
 constexpr int kSmallBlock = 128;                // their threads per block, whatever the tuning's
 
 // conc_set: the set of library streams a concurrent program of this call uses
