@@ -448,7 +448,8 @@ __global__ void __launch_bounds__(32 * kBrickWarps, 16) k_bake_bricks(const Bake
 // Few triangles (few_triangles): one traversal per thread, whose path is shorter than
 // the fixed steps of a brick's search.  What bounds it is the latency of the nodes and
 // triangles of the longest path.  A sample searches within the bound that its source's
-// value gives, so no sites are kept and no scratch is needed.
+// value gives, so no sites are kept and no scratch is needed: a bake that cannot have
+// its scratch takes this too.
 struct ThreadPass {
     int32_t sub;        // > 0: only the samples whose indices are multiples of it
     int32_t own;        // > 0: the source is this grid's own samples at that stride, which are left as they are
@@ -961,6 +962,7 @@ rt_status rt_launch_cascade_bake(const rt_scene* sc, const rt_sdf* sdf, int k, c
     }
     BakeScratch scratch(s);
     const rt_status st = scratch.take(sub_sites_bytes(b.n));
+    if (st == RT_ERR_OOM) return whole_level_by_threads(b, sdf, k, s);
     if (st != RT_OK) return st;
     return launch_two_pass(b, static_cast<int32_t*>(scratch.p), s);
 }
@@ -978,6 +980,7 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
         if (pick_brute(b, method)) return launch_brute(b, s);
         if (few_triangles(b, false)) return launch_threads_two_pass(b, s);
         rt_status st = scratch.take(sub_sites_bytes(b.n));
+        if (st == RT_ERR_OOM) return launch_threads_two_pass(b, s);
         if (st != RT_OK) return st;
         return launch_two_pass(b, static_cast<int32_t*>(scratch.p), s);
     }
@@ -989,7 +992,7 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
         }
         return RT_OK;
     }
-    if (few_triangles(first, true)) {
+    auto by_threads = [&] {
         // coarsest first: each level bounds the next finer one
         for (int k = sdf->levels - 1; k >= 0; --k) {
             BakeArgs b = level_args(sc, sdf, k);
@@ -998,12 +1001,14 @@ rt_status rt_launch_bake(const rt_scene* sc, const rt_sdf* sdf, int32_t method, 
             if (st != RT_OK) return st;
         }
         return RT_OK;
-    }
+    };
+    if (few_triangles(first, true)) return by_threads();
     // coarsest first: each level starts from the nearest triangles of the next
     // coarser one, kept for two levels at a time
     const size_t sub_bytes = sub_sites_bytes(sdf->n);
     const size_t level_bytes = ((size_t)sdf->n[0] * sdf->n[1] * sdf->n[2] * sizeof(int32_t) + 255) & ~(size_t)255;
     rt_status st = scratch.take(sub_bytes + (sdf->levels > 1 ? 2 * level_bytes : 0));
+    if (st == RT_ERR_OOM) return by_threads();
     if (st != RT_OK) return st;
     char* base = static_cast<char*>(scratch.p);
     for (int k = sdf->levels - 1; k >= 0; --k) {
