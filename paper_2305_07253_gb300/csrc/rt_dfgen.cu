@@ -378,7 +378,9 @@ __global__ void __launch_bounds__(kJfaBlock) k_df_jfa(const DfGrid g, const Tris
     const bool on = s < g.count;
     const int64_t s0 = on ? s : 0;
     const int32_t nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int32_t i = (int32_t)(s0 % nx), jk = (int32_t)(s0 / nx), j = jk % ny, k = jk / ny;
+    const int64_t jk = s0 / nx;
+    const int32_t i = (int32_t)(s0 - jk * nx);
+    const int32_t k = jk <= 0x7fffffff ? (int32_t)jk / ny : (int32_t)(jk / ny), j = (int32_t)(jk - (int64_t)k * ny);
     int32_t near[27];
 #pragma unroll
     for (int q = 0; q < 27; ++q) {
