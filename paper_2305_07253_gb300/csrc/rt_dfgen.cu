@@ -15,8 +15,9 @@
 //   2. Jump flooding (Rong & Tan, I3D 2006): steps k = 2^(ceil(log2 n)-1) ...
 //      1; each sample takes the best of the sites of itself and its 26
 //      neighbours at offsets in {-k, 0, k}^3, from the previous step.
-//   3. Fast sweeping as axis sweeps, +x, -x, +y, -y, +z, -z: one thread per
-//      grid line carries the best site along the line.
+//   3. Fast sweeping as axis sweeps, +x, -x, +y, -y, +z, -z: the best site is
+//      carried along each grid line, by a warp (by a thread on lines too long for
+//      its shared memory).
 //   4. The field value is the signed distance to the site triangle (the
 //      exact bake's closest point and pseudonormal sign).
 //
@@ -452,24 +453,11 @@ __global__ void __launch_bounds__(kJfaBlock) k_df_jfa(const DfGrid g, const Tris
 // sequential sweep, since the sweep only writes samples it has passed.
 constexpr int kSweepChunk = 8;
 
-// the grids swept by one launch (all levels of a cascade at once)
-struct SweepPass {
-    DfGrid g[RT_MAX_LEVELS];
-    int32_t* sites[RT_MAX_LEVELS];
-    int64_t first_line[RT_MAX_LEVELS + 1];  // prefix sums of the levels' line counts
-    int32_t count;
-};
-
-__global__ void k_df_sweep(const SweepPass sp, const Tris T, int axis, int dir)
+__global__ void k_df_sweep(const DfGrid g, const Tris T, int32_t* sites, int axis, int dir)
 {
     const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= sp.first_line[sp.count]) return;
-    int l = 0;
-    while (l + 1 < sp.count && t >= sp.first_line[l + 1]) ++l;
-    const DfGrid& g = sp.g[l];
-    int32_t* sites = sp.sites[l];
-    const int64_t line = t - sp.first_line[l];
+    const int64_t line = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (line >= (int64_t)g.n[oa] * g.n[ob]) return;
     const int64_t n[3] = {g.n[0], g.n[1], g.n[2]};
     const int64_t stride[3] = {1, n[0], n[0] * n[1]};
     const int64_t ua = line % n[oa], ub = line / n[oa];
@@ -584,7 +572,7 @@ __device__ __forceinline__ void sweep_line(const DfGrid& g, int32_t ii[3], int a
             const int r = ok ? at(step + lane) : 0;
             float e = 0.f;
             const bool takes = ok && line_offer(g, ii, axis, tri, d2, from, r, carried, e);
-            const bool same = ok && from[r] >= 0 && tri[3 * from[r]].w == tri[3 * carried].w;
+            const bool same = ok && from[r] >= 0 && __float_as_int(tri[3 * from[r]].w) == __float_as_int(tri[3 * carried].w);
             const unsigned stop = __ballot_sync(full, ok && !takes && !same);
             const int end = stop ? __ffs(stop) - 1 : 32;
             __syncwarp();
@@ -796,14 +784,8 @@ rt_status df_build(const rt_scene* sc, const rt_sdf* sdf, const int* lv, int nl,
                     if (st == RT_OK)
                         k_df_sweep_line<<<(unsigned)((lines + warps - 1) / warps), 32 * warps, smem, s>>>(g, T, sites, axis);
                 } else {
-                    SweepPass sp;
-                    memset(&sp, 0, sizeof(sp));
-                    sp.count = 1;
-                    sp.g[0] = g;
-                    sp.sites[0] = sites;
-                    sp.first_line[1] = lines;
                     for (int dir = 1; dir >= -1; dir -= 2)
-                        k_df_sweep<<<(unsigned)((lines + 63) / 64), 64, 0, s>>>(sp, T, axis, dir);
+                        k_df_sweep<<<(unsigned)((lines + 63) / 64), 64, 0, s>>>(g, T, sites, axis, dir);
                 }
             }
         }
