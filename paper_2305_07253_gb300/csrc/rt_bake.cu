@@ -557,10 +557,34 @@ __global__ void k_roll(const void* keep, void* grid, int32_t f16, int32_t n, int
 
 // The copies of a grid that the march reads (layouts: rt_internal.cuh), written in
 // one pass: cell entries for j < ny-1, k < nz-1, and (pairs non-null) x-pairs for
-// i < nx-1.  One thread per sample of a row; a block's threads share one row, so
-// its indices cost one division per block.  Bound by the bytes written: 256^3
-// float32 (67 MB read, 268 + 134 MB written; 69 us at the copy bandwidth).
+// i < nx-1.  A thread takes the samples of kCopyRows successive rows at one i; a block
+// takes a part of long rows, or short rows side by side.  us with one, two, four and
+// eight rows a thread: 256^3 float32 123, 97, 90, 97; 5 x 200^3 float16 326, 244, 193,
+// 175 (blocks of one row of a thread each: 109 and 290, and 277 for 2 x 700 x 700
+// samples, now 10).  Bound by the bytes written: 256^3 float32 (67 MB read, 268 + 134 MB
+// written; 69 us at the copy bandwidth).
 constexpr int kCopyBlock = 128;
+constexpr int kCopyRows = 4;
+
+// how a block's threads lie over rows of nx samples: long rows are cut into equal
+// parts of whole warps
+struct CopyShape {
+    int32_t width, rows, chunks;  // threads beside one another in a row, rows side by side, parts of a row
+};
+static CopyShape copy_shape(int32_t nx)
+{
+    CopyShape c;
+    c.chunks = (nx + kCopyBlock - 1) / kCopyBlock;
+    const int32_t part = (nx + c.chunks - 1) / c.chunks;
+    if (part > 32) {
+        c.width = (part + 31) / 32 * 32;
+    } else {
+        c.width = 2;
+        while (c.width < part) c.width *= 2;
+    }
+    c.rows = kCopyBlock / c.width;
+    return c;
+}
 
 template <class V2>
 struct __align__(2 * sizeof(V2)) Quad {
@@ -574,30 +598,41 @@ __device__ __forceinline__ Quad<float2> quad(float a, float b, float c, float d)
 
 template <class T, class V2, class V4>
 __global__ void __launch_bounds__(kCopyBlock) k_copies(const T* __restrict__ grid, int32_t nx, int32_t ny, int32_t nz,
-                                                       int64_t samples, int64_t entries, int shift,
+                                                       CopyShape shape, int64_t samples, int64_t entries, int shift,
                                                        V4* __restrict__ cells, V2* __restrict__ pairs)
 {
     static_assert(sizeof(V4) == sizeof(Quad<V2>), "one entry is two pairs");
-    const uint32_t chunks = (uint32_t)((nx + kCopyBlock - 1) / kCopyBlock);
-    const uint64_t total = (uint64_t)chunks * (uint64_t)ny * (uint64_t)nz;
+    const uint32_t chunks = (uint32_t)shape.chunks, per = (uint32_t)shape.rows * kCopyRows;
+    const uint64_t rows = (uint64_t)ny * (uint64_t)nz, total = chunks * ((rows + per - 1) / per);
+    const bool wide = ((rows + per) | total) >> 32 != 0;  // (32-bit divisions wherever they suffice)
+    const uint32_t mine = threadIdx.x / (uint32_t)shape.width, lane = threadIdx.x - mine * (uint32_t)shape.width;
     for (uint64_t at = blockIdx.x; at < total; at += gridDim.x) {
-        // (32-bit divisions wherever they suffice)
-        const uint64_t row = total >> 32 ? at / chunks : (uint32_t)at / chunks;
-        const int32_t i = (int32_t)((at - row * chunks) * kCopyBlock + threadIdx.x);
-        const int32_t k = (int32_t)(total >> 32 ? row / (uint32_t)ny : (uint32_t)row / (uint32_t)ny);
-        const int32_t j = (int32_t)(row - (uint64_t)k * (uint32_t)ny);
-        if (i >= nx) continue;
-        const T* g = grid + blockIdx.y * samples + i + (int64_t)nx * (int64_t)row;
-        const T v = g[0];
-        if (pairs && i + 1 < nx) {
-            const Quad<V2> q = quad(v, g[1], v, v);
-            pairs[i + (int64_t)(nx - 1) * (int64_t)row] = q.a;
-        }
-        if (j + 1 < ny && k + 1 < nz) {
-            const Quad<V2> q = quad(v, g[nx], g[(int64_t)nx * ny], g[(int64_t)nx * ny + nx]);
-            const int64_t e = (blockIdx.y * entries + rtdev::cell_slot(i, j, k, nx, ny)) << shift;
-            cells[e] = *reinterpret_cast<const V4*>(&q);
-            if (shift && i > 0) cells[e - 1] = *reinterpret_cast<const V4*>(&q);
+        const uint64_t group = wide ? at / chunks : (uint32_t)at / chunks;
+        const uint64_t row0 = group * per + mine * kCopyRows;
+        const int32_t i = (int32_t)((at - group * chunks) * (uint32_t)shape.width + lane);
+        if (i >= nx || row0 >= rows) continue;
+        int32_t k = (int32_t)(wide ? row0 / (uint32_t)ny : (uint32_t)row0 / (uint32_t)ny);
+        int32_t j = (int32_t)(row0 - (uint64_t)k * (uint32_t)ny);
+#pragma unroll
+        for (int u = 0; u < kCopyRows; ++u) {
+            const int64_t row = (int64_t)row0 + u;
+            if ((uint64_t)row >= rows) break;
+            const T* g = grid + blockIdx.y * samples + i + (int64_t)nx * row;
+            const T v = g[0];
+            if (pairs && i + 1 < nx) {
+                const Quad<V2> q = quad(v, g[1], v, v);
+                pairs[i + (int64_t)(nx - 1) * row] = q.a;
+            }
+            if (j + 1 < ny && k + 1 < nz) {
+                const Quad<V2> q = quad(v, g[nx], g[(int64_t)nx * ny], g[(int64_t)nx * ny + nx]);
+                const int64_t e = (blockIdx.y * entries + i + (int64_t)nx * (row - k)) << shift;  // (rtdev::cell_slot(i, j, k))
+                cells[e] = *reinterpret_cast<const V4*>(&q);
+                if (shift && i > 0) cells[e - 1] = *reinterpret_cast<const V4*>(&q);
+            }
+            if (++j == ny) {
+                j = 0;
+                ++k;
+            }
         }
     }
 }
@@ -606,15 +641,17 @@ __global__ void __launch_bounds__(kCopyBlock) k_copies(const T* __restrict__ gri
 rt_status launch_copies(const void* grid, int32_t dtype, const int32_t n[3], int levels, int shift, void* cells,
                         void* pairs, cudaStream_t s)
 {
-    const int64_t total = (int64_t)((n[0] + kCopyBlock - 1) / kCopyBlock) * n[1] * n[2];
+    const CopyShape shape = copy_shape(n[0]);
+    const int block = shape.width * shape.rows;
+    const int64_t per = shape.rows * kCopyRows, total = shape.chunks * (((int64_t)n[1] * n[2] + per - 1) / per);
     const dim3 blocks((unsigned)(total < 0x7fffffffLL ? total : 0x7fffffffLL), (unsigned)levels);
     const int64_t samples = (int64_t)n[0] * n[1] * n[2], entries = rtdev::cell_count(n[0], n[1], n[2]);
     if (dtype == RT_GRID_F16)
-        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const __half*>(grid), n[0], n[1], n[2], samples, entries, shift,
-                                               static_cast<uint2*>(cells), static_cast<__half2*>(pairs));
+        k_copies<<<blocks, block, 0, s>>>(static_cast<const __half*>(grid), n[0], n[1], n[2], shape, samples, entries, shift,
+                                          static_cast<uint2*>(cells), static_cast<__half2*>(pairs));
     else
-        k_copies<<<blocks, kCopyBlock, 0, s>>>(static_cast<const float*>(grid), n[0], n[1], n[2], samples, entries, shift,
-                                               static_cast<float4*>(cells), static_cast<float2*>(pairs));
+        k_copies<<<blocks, block, 0, s>>>(static_cast<const float*>(grid), n[0], n[1], n[2], shape, samples, entries, shift,
+                                          static_cast<float4*>(cells), static_cast<float2*>(pairs));
     RT_CUDA_TRY(cudaGetLastError());
     return RT_OK;
 }

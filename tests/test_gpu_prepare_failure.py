@@ -13,16 +13,18 @@ MB = 1 << 20
 
 
 def _leave_free(nbytes):
-    """Allocate device memory until at most 32 MB more than nbytes are left; returns what holds it."""
+    """Hold all device memory but nbytes to nbytes + 32 MB.  First everything, so that
+    what idle memory pools keep (an allocation that fails empties them) is held too."""
     torch.cuda.empty_cache()
-    held = []
-    step = 64 << 30
-    while step >= 32 * MB:  # (smaller ones come from larger blocks of the tensor allocator)
-        free = torch.cuda.mem_get_info()[0]
-        if free - step < nbytes:
-            step //= 2
-            continue
-        held.append(torch.empty(step, dtype=torch.uint8, device="cuda"))
+    held = [torch.empty(max(torch.cuda.mem_get_info()[0] - 4096 * MB, 32 * MB), dtype=torch.uint8, device="cuda")]
+    try:
+        while True:
+            held.append(torch.empty(32 * MB, dtype=torch.uint8, device="cuda"))
+    except torch.cuda.OutOfMemoryError:
+        pass
+    while torch.cuda.mem_get_info()[0] < nbytes:
+        held.pop()
+        torch.cuda.empty_cache()
     return held
 
 
