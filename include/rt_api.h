@@ -430,12 +430,12 @@ rt_status rt_trace_combined_backward(const rt_scene* scene, const rt_sdf* sdf, c
  * call (rt_sdf_prepare, rt_sdf_bake, rt_cascade_recenter) writes them.  0: there
  * are none yet, or such a call has been captured into a graph, whose replays write
  * them without the handle's knowledge. */
-rt_status rt_sdf_version(const rt_sdf* sdf, uint64_t* version);
+uint64_t rt_sdf_version(const rt_sdf* sdf);
 
 /* rt_trace_combined_backward for records that a forward call with the same rays
  * and params and refine_root = 1 found when rt_sdf_version gave `version`, the
  * copies and the grid holding the same values then.  While that is still the
- * number, the root is the record's t and the ray is not marched again (4.6 times
+ * number, the root is the record's t and the ray is not marched again (4.4 times
  * as fast); otherwise (another number, 0, a stream that is being captured) each
  * ray is, as by rt_trace_combined_backward. */
 rt_status rt_trace_combined_backward_at(const rt_scene* scene, const rt_sdf* sdf, uint64_t version,

@@ -112,7 +112,6 @@ def lib() -> ctypes.CDLL:
             "rt_trace_batches": [P, P, P, i32, P],
             "rt_trace_combined_backward": [P, P, P, i64, P, P, P, P, P],
             "rt_trace_combined_backward_at": [P, P, ctypes.c_uint64, P, i64, P, P, P, P, P],
-            "rt_sdf_version": [P, P],
             "rt_cascade_create": [P, i32, i32, i32, ctypes.c_float, P, P],
             "rt_cascade_recenter": [P, P, P, P, P],
             "rt_cascade_level": [P, i32, P, P],
@@ -126,6 +125,7 @@ def lib() -> ctypes.CDLL:
             f.restype = st
         L.rt_last_error.restype = ctypes.c_char_p
         L.rt_version.restype = ctypes.c_char_p
+        L.rt_sdf_version.argtypes, L.rt_sdf_version.restype = [P], ctypes.c_uint64
         _lib = L
         return L
 
@@ -418,9 +418,7 @@ def rt_trace_combined_timed(scene: Scene | None, sdf: Sdf | None, rays: torch.Te
 
 def rt_sdf_version(sdf: Sdf) -> int:
     """Number of the copies of the grid that traces read (0: none, or not known)."""
-    v = ctypes.c_uint64()
-    _check(lib().rt_sdf_version(sdf.handle, ctypes.byref(v)))
-    return v.value
+    return lib().rt_sdf_version(sdf.handle)
 
 
 def rt_trace_combined_backward(scene: Scene | None, sdf: Sdf, rays: torch.Tensor, params: rt_split_params,

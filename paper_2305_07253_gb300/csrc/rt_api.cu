@@ -668,12 +668,7 @@ extern "C" rt_status rt_trace_combined_counted(const rt_scene* sc, const rt_sdf*
     return trace_common(sc, sdf, rays, n, params, hits, counters, stream);
 }
 
-extern "C" rt_status rt_sdf_version(const rt_sdf* sdf, uint64_t* version)
-{
-    if (!sdf || !version) return rt_fail(RT_ERR_INVALID_ARG, "null argument");
-    *version = sdf->replayed ? 0 : sdf->version;
-    return RT_OK;
-}
+extern "C" uint64_t rt_sdf_version(const rt_sdf* sdf) { return !sdf || sdf->replayed ? 0 : sdf->version; }
 
 extern "C" rt_status rt_trace_combined_backward(const rt_scene* sc, const rt_sdf* sdf, const rt_ray* rays, int64_t n,
                                                 const rt_split_params* params, const rt_hit* hits,
