@@ -343,22 +343,24 @@ rt_status device_info(DeviceInfo*& out)
     if (dev < 0 || dev >= 64) return rt_fail(RT_ERR_INVALID_ARG, "device %d out of range", dev);
     std::lock_guard<std::mutex> lk(g_mu);
     DeviceInfo& d = g_dev[dev];
-    if (d.sms == 0) {
-        RT_CUDA_TRY(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev));
+    if (d.sms == 0) {  // (set last: a failed set-up is tried again)
+        int sms = 0;
+        RT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.handleTypes = cudaMemHandleTypeNone;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        RT_CUDA_TRY(cudaMemPoolCreate(&d.pool, &props));
+        if (!d.pool) RT_CUDA_TRY(cudaMemPoolCreate(&d.pool, &props));
         // keep freed scratch in the pool between calls instead of returning it
         uint64_t keep = ~0ull;
         RT_CUDA_TRY(cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep));
         // builds and bakes on many streams at once hold more for a while; what exceeds
         // this goes back at the next synchronisation
-        RT_CUDA_TRY(cudaMemPoolCreate(&d.scratch, &props));
+        if (!d.scratch) RT_CUDA_TRY(cudaMemPoolCreate(&d.scratch, &props));
         keep = 2 * kScratchKept;
         RT_CUDA_TRY(cudaMemPoolSetAttribute(d.scratch, cudaMemPoolAttrReleaseThreshold, &keep));
+        d.sms = sms;
     }
     out = &d;
     return RT_OK;
