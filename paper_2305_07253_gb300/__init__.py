@@ -479,7 +479,7 @@ class SdfHitDistance(torch.autograd.Function):
         p = rt_split_params.from_buffer_copy(params)
         p.refine_root = 1
         hits = rt_trace_combined(scene, sdf, rays, p)
-        t = hit_fields(hits)["t"].clone()
+        t = hits[:, 0].view(torch.float32).clone()
         ctx.save_for_backward(rays, hits)
         ctx.scene, ctx.sdf, ctx.params = scene, sdf, p
         ctx.version = rt_sdf_version(sdf)
